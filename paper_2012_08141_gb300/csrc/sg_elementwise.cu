@@ -47,6 +47,7 @@ constexpr int kEwThreads = 128;
 template <int L>
 __global__ void __launch_bounds__(kEwThreads, 8) k_ew(DevGrid g, EwProgram prog)
 {
+    chained_entry();
     constexpr int V = L * L * L, Q = V / 8, LG2 = (L == 8) ? 3 : 2;
     extern __shared__ float4 s_reg[];  // [n_slots][2][kEwThreads]
     __shared__ double s_red[kEwThreads / 32];
@@ -149,8 +150,8 @@ void launch_ew(const DevGrid &g, cudaStream_t s, const EwProgram &prog, const La
     for (int k = 0; k < p.n_slots; ++k) p.fp[k] = g.field[p.field[k]];
     const int ns = p.n_slots < 1 ? 1 : p.n_slots;
     const size_t smem = sizeof(float4) * 2 * kEwThreads * ns;
-    if (g.L == 8) k_ew<8><<<ew_ctas<8>(lc.num_sms, ns), kEwThreads, smem, s>>>(g, p);
-    else k_ew<4><<<ew_ctas<4>(lc.num_sms, ns), kEwThreads, smem, s>>>(g, p);
+    if (g.L == 8) launch_chained(k_ew<8>, ew_ctas<8>(lc.num_sms, ns), kEwThreads, smem, s, g, p);
+    else launch_chained(k_ew<4>, ew_ctas<4>(lc.num_sms, ns), kEwThreads, smem, s, g, p);
 }
 
 }  // namespace sg

@@ -231,6 +231,7 @@ __global__ void __launch_bounds__(256, L == 4 ? 3 : 2) k_g2p2g(DevGrid src, DevG
                                                float *__restrict__ v, float dt, int f_vel0, float pmass, int f_mass,
                                                int f_mom0, bool pair)
 {
+    chained_entry();
     using S = G2P2GSmem<L>;
     constexpr int LG2 = (L == 8) ? 3 : 2, BD = S::BD, C1 = S::C1, NC = S::NC, ND = S::ND;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -426,7 +427,7 @@ void launch_g2p2g_L(const DevGrid &src, const DevGrid &dst, const DevGrid &bins,
         resident.store(per, std::memory_order_relaxed);
     }
     const int ctas = per * num_sms;
-    k_g2p2g<L><<<ctas, 256, bytes, s>>>(src, dst, bins.bin_list, bins.bin_off, bins.bin_count, bins.perm,
+    launch_chained(k_g2p2g<L>, ctas, 256, bytes, s, src, dst, bins.bin_list, bins.bin_off, bins.bin_count, bins.perm,
                                          &bins.ctrl->bins_used, x, v, dt, f_vel0, pmass, f_mass, f_mom0, pair);
 }
 

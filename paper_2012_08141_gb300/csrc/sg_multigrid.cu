@@ -35,6 +35,7 @@ __global__ void k_restrict_mark(DevGrid fine, DevGrid coarse)
 template <int L, bool ACTIVATE>
 __global__ void __launch_bounds__(256) k_restrict(DevGrid fine, DevGrid coarse, int f_src, int f_dst, float w)
 {
+    chained_entry();
     constexpr int H = L / 2, NV = H * H * H, G = NV < 32 ? NV : 32, PER = NV / G, LG2 = (L == 8) ? 3 : 2;
     const int n = fine.ctrl->list_n;
     const int Rf = fine.R, Rc = coarse.R;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(256) k_restrict(DevGrid fine, DevGrid coarse, 
 template <int L>
 __global__ void __launch_bounds__(256) k_prolong(DevGrid coarse, DevGrid fine, int f_src, int f_dst, float w)
 {
+    chained_entry();
     constexpr int LG2 = (L == 8) ? 3 : 2, V = L * L * L;
     const long long n = fine.ctrl->list_n;
     const int Rf = fine.R, Rc = coarse.R;
@@ -116,6 +118,7 @@ __global__ void __launch_bounds__(256) k_prolong(DevGrid coarse, DevGrid fine, i
 // move as float4s.  Each active voxel takes the same fma as in k_prolong.
 __global__ void __launch_bounds__(256) k_prolong8(DevGrid coarse, DevGrid fine, int f_src, int f_dst, float w)
 {
+    chained_entry();
     const long long n = fine.ctrl->list_n;
     const int Rf = fine.R, Rc = coarse.R;
     const float *__restrict__ y = coarse.field[f_src];
@@ -158,6 +161,7 @@ __global__ void __launch_bounds__(256) k_prolong8(DevGrid coarse, DevGrid fine, 
 template <bool ACTIVATE>
 __global__ void __launch_bounds__(256) k_restrict8(DevGrid fine, DevGrid coarse, int f_src, int f_dst, float w)
 {
+    chained_entry();
     const long long n = fine.ctrl->list_n;
     const int Rf = fine.R, Rc = coarse.R;
     const float *__restrict__ x = fine.field[f_src];
@@ -214,11 +218,11 @@ void launch_restrict(const DevGrid &fine, const DevGrid &coarse, cudaStream_t s,
 {
     const int ctas = lc.num_sms * 8;
     if (fine.L == 8) {
-        if (activate) k_restrict8<true><<<ctas, 256, 0, s>>>(fine, coarse, f_src, f_dst, w);
-        else k_restrict8<false><<<ctas, 256, 0, s>>>(fine, coarse, f_src, f_dst, w);
+        if (activate) launch_chained(k_restrict8<true>, ctas, 256, 0, s, fine, coarse, f_src, f_dst, w);
+        else launch_chained(k_restrict8<false>, ctas, 256, 0, s, fine, coarse, f_src, f_dst, w);
     } else {
-        if (activate) k_restrict<4, true><<<ctas, 256, 0, s>>>(fine, coarse, f_src, f_dst, w);
-        else k_restrict<4, false><<<ctas, 256, 0, s>>>(fine, coarse, f_src, f_dst, w);
+        if (activate) launch_chained(k_restrict<4, true>, ctas, 256, 0, s, fine, coarse, f_src, f_dst, w);
+        else launch_chained(k_restrict<4, false>, ctas, 256, 0, s, fine, coarse, f_src, f_dst, w);
     }
 }
 
@@ -226,8 +230,8 @@ void launch_prolong(const DevGrid &coarse, const DevGrid &fine, cudaStream_t s, 
                     const LaunchCfg &lc)
 {
     const int ctas = lc.num_sms * 8;
-    if (fine.L == 8) k_prolong8<<<ctas, 256, 0, s>>>(coarse, fine, f_src, f_dst, w);
-    else k_prolong<4><<<ctas, 256, 0, s>>>(coarse, fine, f_src, f_dst, w);
+    if (fine.L == 8) launch_chained(k_prolong8, ctas, 256, 0, s, coarse, fine, f_src, f_dst, w);
+    else launch_chained(k_prolong<4>, ctas, 256, 0, s, coarse, fine, f_src, f_dst, w);
 }
 
 }  // namespace sg

@@ -14,6 +14,7 @@ namespace sg {
 // Grid update over the active nodes of the listed leaves.
 __global__ void __launch_bounds__(256) k_grid_update(DevGrid g, int f_mass, int f_mom0, float dt, float gz, int bound)
 {
+    chained_entry();
     const long long n = g.ctrl->list_n;
     const int L = g.L, lg2 = g.lg2, R = g.R, N = g.N, V = L * L * L;
     float *fm = g.field[f_mass];
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(256) k_grid_update(DevGrid g, int f_mass, int 
 void launch_grid_update(const DevGrid &g, cudaStream_t s, int f_mass, int f_mom0, float dt, float gz, int bound,
                         const LaunchCfg &lc)
 {
-    k_grid_update<<<lc.num_sms * 8, 256, 0, s>>>(g, f_mass, f_mom0, dt, gz, bound);
+    launch_chained(k_grid_update, lc.num_sms * 8, 256, 0, s, g, f_mass, f_mom0, dt, gz, bound);
 }
 
 // G2P in input order, every node read from the grid.
@@ -55,6 +56,7 @@ template <bool APIC>
 __global__ void __launch_bounds__(256) k_g2p(DevGrid g, float *__restrict__ x, float *__restrict__ v,
                                              float *__restrict__ C, long long n, float dt, int f_mom0)
 {
+    chained_entry();
     const float *f0 = g.field[f_mom0], *f1 = g.field[f_mom0 + 1], *f2 = g.field[f_mom0 + 2];
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         const float3 xp = make_float3(x[3 * p], x[3 * p + 1], x[3 * p + 2]);
@@ -93,6 +95,7 @@ template <int L, bool APIC>
 __global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(DevGrid g, float *__restrict__ x, float *__restrict__ v,
                                                        float *__restrict__ C, float dt, int f_mom0)
 {
+    chained_entry();
     constexpr int B = L + 2, NB = B * B * B;  // nodes o .. o + L + 1 of the bin's leaf o
     __shared__ float4 s_u[NB];
     __shared__ float s_words[8][32 * (APIC ? 9 : 3)];
@@ -165,8 +168,7 @@ void launch_g2p(const DevGrid &g, cudaStream_t s, float *x, float *v, float *C, 
 {
     if (n <= 0) return;
     if (binned) {
-#define SG_G2PB(LL, AP) k_g2p_binned<LL, AP><<<resident_ctas(k_g2p_binned<LL, AP>, lc.num_sms), 256, 0, s>>>( \
-        g, x, v, C, dt, f_mom0)
+#define SG_G2PB(LL, AP) launch_chained(k_g2p_binned<LL, AP>, resident_ctas(k_g2p_binned<LL, AP>, lc.num_sms), 256, 0, s, g, x, v, C, dt, f_mom0)
         if (C) {
             if (g.L == 4) SG_G2PB(4, true);
             else SG_G2PB(8, true);
@@ -179,8 +181,8 @@ void launch_g2p(const DevGrid &g, cudaStream_t s, float *x, float *v, float *C, 
     }
     long long blocks = (n + 255) / 256;
     if (blocks > 1 << 20) blocks = 1 << 20;
-    if (C) k_g2p<true><<<(unsigned)blocks, 256, 0, s>>>(g, x, v, C, n, dt, f_mom0);
-    else k_g2p<false><<<(unsigned)blocks, 256, 0, s>>>(g, x, v, C, n, dt, f_mom0);
+    if (C) launch_chained(k_g2p<true>, (unsigned)blocks, 256, 0, s, g, x, v, C, n, dt, f_mom0);
+    else launch_chained(k_g2p<false>, (unsigned)blocks, 256, 0, s, g, x, v, C, n, dt, f_mom0);
 }
 
 }  // namespace sg
@@ -235,6 +237,7 @@ __device__ __forceinline__ long long p2g_key_of(const float *__restrict__ x, lon
 // for the order passes, which then read keys in order instead of positions.
 __global__ void k_p2g_bin(DevGrid g, const float *__restrict__ x, long long n)
 {
+    chained_entry();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         const long long key = p2g_key_of(x, p, g.N, g.lg2, g.R);
         g.perm_key[p] = key;
@@ -247,6 +250,7 @@ __global__ void k_p2g_bin(DevGrid g, const float *__restrict__ x, long long n)
 // one atomic per distinct key in the warp.
 __global__ void k_p2g_rebin(DevGrid g, const float *__restrict__ x, long long n)
 {
+    chained_entry();
     const int lane = lane_id();
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const long long key = p2g_key_of(x, g.perm[q], g.N, g.lg2, g.R);
@@ -261,6 +265,7 @@ __global__ void k_p2g_rebin(DevGrid g, const float *__restrict__ x, long long n)
 // the directions of its reach class) for allocation.
 __global__ void __launch_bounds__(256) k_bin_scan_tiles(DevGrid g, long long nkeys)
 {
+    chained_entry();
     __shared__ int s_w[8];
     const long long base = (long long)blockIdx.x * kBinTile;
     const long long nleaf_keys = nkeys - 1;  // the last key holds particles outside the domain
@@ -294,6 +299,7 @@ __global__ void __launch_bounds__(256) k_bin_scan_tiles(DevGrid g, long long nke
 // Exclusive scan of the tile sums by one CTA (in place).
 __global__ void __launch_bounds__(1024) k_bin_scan_top(DevGrid g, int ntiles)
 {
+    chained_entry();
     __shared__ int s_w[32];
     __shared__ int s_carry;
     if (threadIdx.x == 0) s_carry = 0;
@@ -321,6 +327,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan_top(DevGrid g, int ntiles)
 // insertion cursor (= offset), bin_off keeps the offset.
 __global__ void __launch_bounds__(256) k_bin_scan_apply(DevGrid g, long long nbins)
 {
+    chained_entry();
     __shared__ int s_w[8];
     const long long base = (long long)blockIdx.x * kBinTile + threadIdx.x * 4;
     int v[4], t = 0;
@@ -361,6 +368,7 @@ __global__ void __launch_bounds__(256) k_bin_scan_apply(DevGrid g, long long nbi
 
 __global__ void k_p2g_perm(DevGrid g, long long n)
 {
+    chained_entry();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < n; p += (long long)gridDim.x * blockDim.x) {
         const int pos = atomicAdd(&g.bin_count[g.perm_key[p]], 1);
         g.perm[pos] = (int)p;
@@ -371,6 +379,7 @@ __global__ void k_p2g_perm(DevGrid g, long long n)
 // cursor atomics, as in k_p2g_rebin).
 __global__ void k_p2g_reperm(DevGrid g, long long n)
 {
+    chained_entry();
     const int lane = lane_id();
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n; q += (long long)gridDim.x * blockDim.x) {
         const int p = g.perm[q];
@@ -406,6 +415,7 @@ template <int L, bool APIC>
 __global__ void __launch_bounds__(256) k_p2g_gather(DevGrid g, const float *__restrict__ x, const float *__restrict__ v,
                                                     const float *__restrict__ C, float pmass, int f_mass, int f_mom0)
 {
+    chained_entry();
     constexpr int B = L + 2, NB = B * B * B, LG2 = (L == 8) ? 3 : 2;
     constexpr int C1 = L + 2, NC = C1 * C1 * C1;  // shifted base cells
     constexpr int CAP = (L == 8) ? 256 : (APIC ? 512 : 1024);  // staged particles per chunk
@@ -625,24 +635,23 @@ int launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v
     int launches = 0;
     cudaMemsetAsync(g.bin_count, 0, sizeof(int32_t) * nscan, s);
     cudaMemsetAsync(&g.ctrl->bins_used, 0, sizeof(int32_t), s);
-    if (rebin) k_p2g_rebin<<<(unsigned)pblocks, 256, 0, s>>>(g, x, n);
-    else k_p2g_bin<<<(unsigned)pblocks, 256, 0, s>>>(g, x, n);
-    k_bin_scan_tiles<<<ntiles, 256, 0, s>>>(g, nscan);
+    if (rebin) launch_chained(k_p2g_rebin, (unsigned)pblocks, 256, 0, s, g, x, n);
+    else launch_chained(k_p2g_bin, (unsigned)pblocks, 256, 0, s, g, x, n);
+    launch_chained(k_bin_scan_tiles, ntiles, 256, 0, s, g, nscan);
     launch_alloc_needed(g, s);
-    k_bin_scan_top<<<1, 1024, 0, s>>>(g, ntiles);
-    k_bin_scan_apply<<<ntiles, 256, 0, s>>>(g, nscan);
+    launch_chained(k_bin_scan_top, 1, 1024, 0, s, g, ntiles);
+    launch_chained(k_bin_scan_apply, ntiles, 256, 0, s, g, nscan);
     launches += 5;
     if (rebin) {
-        k_p2g_reperm<<<(unsigned)pblocks, 256, 0, s>>>(g, n);
+        launch_chained(k_p2g_reperm, (unsigned)pblocks, 256, 0, s, g, n);
         int32_t *t = g.perm;  // the new order is now the current one
         g.perm = g.perm_alt;
         g.perm_alt = t;
     } else {
-        k_p2g_perm<<<(unsigned)pblocks, 256, 0, s>>>(g, n);
+        launch_chained(k_p2g_perm, (unsigned)pblocks, 256, 0, s, g, n);
     }
     ++launches;
-#define SG_GATHER(LL, AP) k_p2g_gather<LL, AP><<<resident_ctas(k_p2g_gather<LL, AP>, lc.num_sms), 256, 0, s>>>( \
-        g, x, v, C, pmass, f_mass, f_mom0)
+#define SG_GATHER(LL, AP) launch_chained(k_p2g_gather<LL, AP>, resident_ctas(k_p2g_gather<LL, AP>, lc.num_sms), 256, 0, s, g, x, v, C, pmass, f_mass, f_mom0)
     if (C) {
         if (g.L == 4) SG_GATHER(4, true);
         else SG_GATHER(8, true);

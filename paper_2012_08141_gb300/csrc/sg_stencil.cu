@@ -55,6 +55,7 @@ __device__ __forceinline__ void check_activation_row(const DevGrid &g, int slot,
 template <bool CHECK>
 __global__ void __launch_bounds__(kStageThreads) k_clear(DevGrid g, int dst)
 {
+    chained_entry();
     const int n = g.ctrl->list_n;
     float *out = g.field[dst];
     for (int e = blockIdx.x; e < n; e += gridDim.x) {
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(kStageThreads) k_clear(DevGrid g, int dst)
 
 __global__ void __launch_bounds__(kStageThreads) k_sum(DevGrid g, int src, int slot_out)
 {
+    chained_entry();
     __shared__ double s_red[kStageThreads / 32];
     const int n = g.ctrl->list_n;
     const int V4 = (g.L * g.L * g.L) >> 2;
@@ -361,6 +363,7 @@ __device__ __forceinline__ float tree_read(const DevGrid &g, const float *x, int
 template <int OP, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(256) k_generic(DevGrid g, int src, int dst, float coef, int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[8];
     const int n = g.ctrl->list_n;
     const int L = g.L, lg2 = g.lg2, V = L * L * L, R = g.R;
@@ -436,11 +439,11 @@ void launch_clear(const DevGrid &g, cudaStream_t s, int dst, int check_act, cons
 {
     const int ctas = stencil_persistent_ctas(lc.num_sms, 2);
     if (g.L == 8) {
-        if (check_act) k_clear<true><<<ctas, kStageThreads, 0, s>>>(g, dst);
-        else k_clear<false><<<ctas, kStageThreads, 0, s>>>(g, dst);
+        if (check_act) launch_chained(k_clear<true>, ctas, kStageThreads, 0, s, g, dst);
+        else launch_chained(k_clear<false>, ctas, kStageThreads, 0, s, g, dst);
     } else {
-        if (check_act) k_generic<0, true, false><<<ctas, 256, 0, s>>>(g, dst, dst, 0.f, 0);
-        else k_generic<0, false, false><<<ctas, 256, 0, s>>>(g, dst, dst, 0.f, 0);
+        if (check_act) launch_chained(k_generic<0, true, false>, ctas, 256, 0, s, g, dst, dst, 0.f, 0);
+        else launch_chained(k_generic<0, false, false>, ctas, 256, 0, s, g, dst, dst, 0.f, 0);
     }
 }
 
@@ -463,11 +466,11 @@ static void launch_single(const DevGrid &g, cudaStream_t s, int src, int dst, fl
     } else {
         const int ctas = stencil_persistent_ctas(lc.num_sms, 3);
         if (check_act) {
-            if (sum) k_generic<OP, true, true><<<ctas, 256, 0, s>>>(g, src, dst, coef, sum_slot);
-            else k_generic<OP, true, false><<<ctas, 256, 0, s>>>(g, src, dst, coef, sum_slot);
+            if (sum) launch_chained(k_generic<OP, true, true>, ctas, 256, 0, s, g, src, dst, coef, sum_slot);
+            else launch_chained(k_generic<OP, true, false>, ctas, 256, 0, s, g, src, dst, coef, sum_slot);
         } else {
-            if (sum) k_generic<OP, false, true><<<ctas, 256, 0, s>>>(g, src, dst, coef, sum_slot);
-            else k_generic<OP, false, false><<<ctas, 256, 0, s>>>(g, src, dst, coef, sum_slot);
+            if (sum) launch_chained(k_generic<OP, false, true>, ctas, 256, 0, s, g, src, dst, coef, sum_slot);
+            else launch_chained(k_generic<OP, false, false>, ctas, 256, 0, s, g, src, dst, coef, sum_slot);
         }
     }
 }
@@ -515,7 +518,7 @@ void launch_diffuse_box(const DevGrid &g, cudaStream_t s, int src, int tmp, int 
 void launch_sum(const DevGrid &g, cudaStream_t s, int src, int sum_slot, const LaunchCfg &lc)
 {
     const int ctas = stencil_persistent_ctas(lc.num_sms, 2);
-    k_sum<<<ctas, kStageThreads, 0, s>>>(g, src, sum_slot);
+    launch_chained(k_sum, ctas, kStageThreads, 0, s, g, src, sum_slot);
 }
 
 }  // namespace sg

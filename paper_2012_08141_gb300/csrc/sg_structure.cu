@@ -49,6 +49,7 @@ template <int L>
 __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2_, long long hi2_, int strict, int tube,
                                                         int cpw, uint32_t fill_mask)
 {
+    chained_entry();
     constexpr int LG2 = (L == 8) ? 3 : 2, W = L * L * L / 32;
     constexpr int kMaxW = 16;  // mask words of an 8^3 leaf
     __shared__ uint32_t s_bits[8][32][kMaxW];  // per warp: the mask words of its chunk's cells
@@ -186,8 +187,8 @@ void launch_activate_shell(const DevGrid &g, cudaStream_t s, long long lo2, long
     const long long nr = (long long)g.R * g.R * g.R;
     int cpw, ctas;
     activate_shape(nr, cpw, ctas);
-    if (g.L == 8) k_activate_shell<8><<<ctas, 256, 0, s>>>(g, lo2, hi2, strict, 0, cpw, fill_mask);
-    else k_activate_shell<4><<<ctas, 256, 0, s>>>(g, lo2, hi2, strict, 0, cpw, fill_mask);
+    if (g.L == 8) launch_chained(k_activate_shell<8>, ctas, 256, 0, s, g, lo2, hi2, strict, 0, cpw, fill_mask);
+    else launch_chained(k_activate_shell<4>, ctas, 256, 0, s, g, lo2, hi2, strict, 0, cpw, fill_mask);
 }
 
 void launch_activate_tube(const DevGrid &g, cudaStream_t s, long long lo2, long long hi2, uint32_t fill_mask)
@@ -195,8 +196,8 @@ void launch_activate_tube(const DevGrid &g, cudaStream_t s, long long lo2, long 
     const long long nr = (long long)g.R * g.R * g.R;
     int cpw, ctas;
     activate_shape(nr, cpw, ctas);
-    if (g.L == 8) k_activate_shell<8><<<ctas, 256, 0, s>>>(g, lo2, hi2, 0, 1, cpw, fill_mask);
-    else k_activate_shell<4><<<ctas, 256, 0, s>>>(g, lo2, hi2, 0, 1, cpw, fill_mask);
+    if (g.L == 8) launch_chained(k_activate_shell<8>, ctas, 256, 0, s, g, lo2, hi2, 0, 1, cpw, fill_mask);
+    else launch_chained(k_activate_shell<4>, ctas, 256, 0, s, g, lo2, hi2, 0, 1, cpw, fill_mask);
 }
 
 // ---------------------------------------------------------------------------
@@ -234,6 +235,7 @@ void launch_mark_coords(const DevGrid &g, cudaStream_t s, const int32_t *xyz, lo
 constexpr int kAllocCells = 128;
 __global__ void __launch_bounds__(256) k_alloc_needed(DevGrid g, uint32_t fill_mask)
 {
+    chained_entry();
     __shared__ int s_slot[kAllocCells];
     __shared__ int s_n;
     const long long nr = (long long)g.R * g.R * g.R;
@@ -299,7 +301,7 @@ void launch_alloc_needed(const DevGrid &g, cudaStream_t s, uint32_t fill_mask)
     const long long nr = (long long)g.R * g.R * g.R;
     long long blocks = (nr + kAllocCells - 1) / kAllocCells;
     if (blocks > 4096) blocks = 4096;
-    k_alloc_needed<<<(unsigned)blocks, 256, 0, s>>>(g, fill_mask);
+    launch_chained(k_alloc_needed, (unsigned)blocks, 256, 0, s, g, fill_mask);
 }
 
 __global__ void k_setbits_coords(DevGrid g, const int32_t *__restrict__ xyz, long long n)
@@ -338,6 +340,7 @@ void launch_setbits_coords(const DevGrid &g, cudaStream_t s, const int32_t *xyz,
 // ---------------------------------------------------------------------------
 __global__ void k_deactivate_all(DevGrid g)
 {
+    chained_entry();
     const long long nr = (long long)g.R * g.R * g.R;
     for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < nr; b += (long long)gridDim.x * blockDim.x)
         g.root[b] = -1;
@@ -353,7 +356,7 @@ void launch_deactivate_all(const DevGrid &g, cudaStream_t s)
     const long long nr = (long long)g.R * g.R * g.R;
     long long blocks = (nr + 255) / 256;
     if (blocks > 2048) blocks = 2048;
-    k_deactivate_all<<<(unsigned)blocks, 256, 0, s>>>(g);
+    launch_chained(k_deactivate_all, (unsigned)blocks, 256, 0, s, g);
 }
 
 // Restore a saved structure (checkpoint): one warp per saved leaf e takes
@@ -415,6 +418,7 @@ constexpr unsigned long long kTestWaitLimitNs = 200000000ull;   // 0.2 s
 __global__ void __launch_bounds__(kListThreads) k_listgen(DevGrid g, int force, unsigned long long call_idx,
                                                           int num_tiles, int test_wait)
 {
+    chained_entry();
     __shared__ int s_tile, s_skip, s_prefix;
     __shared__ int s_wsum[kListThreads / 32];
     __shared__ uint32_t s_cells[kListTile];  // listed cells' (i, j, k), 10 bits each (R <= 1024)
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(kListThreads) k_listgen(DevGrid g, int force, 
 void launch_listgen(const DevGrid &g, cudaStream_t s, int force, unsigned long long call_idx, int num_tiles,
                     int test_wait)
 {
-    k_listgen<<<num_tiles, kListThreads, 0, s>>>(g, force, call_idx, num_tiles, test_wait);
+    launch_chained(k_listgen, num_tiles, kListThreads, 0, s, g, force, call_idx, num_tiles, test_wait);
 }
 
 // ---------------------------------------------------------------------------
@@ -557,6 +561,7 @@ void launch_listgen(const DevGrid &g, cudaStream_t s, int force, unsigned long l
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_region_masks(DevGrid g, int group_axis, unsigned long long call)
 {
+    chained_entry();
     const long long n = g.ctrl->list_n;
     const uint8_t *mb = reinterpret_cast<const uint8_t *>(g.mask);
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n * 40; q += (long long)gridDim.x * blockDim.x) {
@@ -688,7 +693,7 @@ void launch_region_masks(const DevGrid &g, cudaStream_t s, const LaunchCfg &lc, 
                          unsigned long long call)
 {
     if (group_axis != kGroupNone) cudaMemsetAsync(&g.ctrl->rr_ticket, 0, sizeof(uint32_t), s);
-    k_region_masks<<<lc.num_sms * 4, 256, 0, s>>>(g, group_axis, call);
+    launch_chained(k_region_masks, lc.num_sms * 4, 256, 0, s, g, group_axis, call);
 }
 
 // ---------------------------------------------------------------------------
@@ -724,6 +729,7 @@ __device__ __forceinline__ float hash24(unsigned long long z)
 template <int L>
 __global__ void __launch_bounds__(256, 6) k_fill_hash(DevGrid g, int f, unsigned long long seed)
 {
+    chained_entry();
     constexpr int LG2 = (L == 8) ? 3 : 2, V4 = L * L * L / 4, G = V4 < 32 ? V4 : 32, W = L * L * L / 32;
     const long long n = g.ctrl->list_n;
     const int R = g.R, r0 = threadIdx.x % G;
@@ -751,8 +757,8 @@ __global__ void __launch_bounds__(256, 6) k_fill_hash(DevGrid g, int f, unsigned
 
 void launch_fill_hash(const DevGrid &g, cudaStream_t s, int f, unsigned long long seed, const LaunchCfg &lc)
 {
-    if (g.L == 8) k_fill_hash<8><<<lc.num_sms * 6, 256, 0, s>>>(g, f, seed);
-    else k_fill_hash<4><<<lc.num_sms * 6, 256, 0, s>>>(g, f, seed);
+    if (g.L == 8) launch_chained(k_fill_hash<8>, lc.num_sms * 6, 256, 0, s, g, f, seed);
+    else launch_chained(k_fill_hash<4>, lc.num_sms * 6, 256, 0, s, g, f, seed);
 }
 
 // ---------------------------------------------------------------------------
@@ -921,6 +927,7 @@ __device__ __forceinline__ long long packed_pos(const DevGrid &g, long long e, i
 __global__ void k_scatter_active(DevGrid g, int f, const float *__restrict__ src, long long total,
                                  const long long *__restrict__ off, const long long *__restrict__ tsum)
 {
+    chained_entry();
     const long long n = g.ctrl->list_n;
     const int V4 = (g.L * g.L * g.L) >> 2;
     float4 *dst = reinterpret_cast<float4 *>(g.field[f]);
@@ -952,6 +959,7 @@ __global__ void __launch_bounds__(256) k_gather_active(DevGrid g, int f, float *
                                                        const long long *__restrict__ off,
                                                        const long long *__restrict__ tsum)
 {
+    chained_entry();
     constexpr int V = L * L * L, W = V / 32, CAP = 4096, T = CAP / V;
     __shared__ float s_val[CAP];
     const long long n = g.ctrl->list_n;
@@ -994,14 +1002,14 @@ __global__ void __launch_bounds__(256) k_gather_active(DevGrid g, int f, float *
 void launch_scatter_active(const DevGrid &g, cudaStream_t s, int f, const float *src, long long total,
                            const long long *off, const long long *tsum, const LaunchCfg &lc)
 {
-    k_scatter_active<<<lc.num_sms * 4, 256, 0, s>>>(g, f, src, total, off, tsum);
+    launch_chained(k_scatter_active, lc.num_sms * 4, 256, 0, s, g, f, src, total, off, tsum);
 }
 
 void launch_gather_active(const DevGrid &g, cudaStream_t s, int f, float *out, long long total, const long long *off,
                           const long long *tsum, const LaunchCfg &lc)
 {
-    if (g.L == 8) k_gather_active<8><<<lc.num_sms * 4, 256, 0, s>>>(g, f, out, total, off, tsum);
-    else k_gather_active<4><<<lc.num_sms * 4, 256, 0, s>>>(g, f, out, total, off, tsum);
+    if (g.L == 8) launch_chained(k_gather_active<8>, lc.num_sms * 4, 256, 0, s, g, f, out, total, off, tsum);
+    else launch_chained(k_gather_active<4>, lc.num_sms * 4, 256, 0, s, g, f, out, total, off, tsum);
 }
 
 // Active voxels of the listed leaves: popcount of their mask words.

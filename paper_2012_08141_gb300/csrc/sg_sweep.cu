@@ -439,6 +439,7 @@ template <bool STORE_T, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(kSweepThreads, 3) k_sweep_columns(DevGrid g, int src, int tmp, int dst, float coef,
                                                                    int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[kSweepThreads / 32];
     const long long cap3 = g.cap * 3;
     const int c3 = g.col_cnt[2], c2 = g.col_cnt[1], c1 = g.col_cnt[0];
@@ -603,6 +604,7 @@ template <bool STORE_T, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(kSweepThreads, 4) k_sweep_jruns(DevGrid g, int src, int tmp, int dst, float coef,
                                                                  int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[kSweepThreads / 32];
     const int c3 = g.col_cnt[2], c2 = g.col_cnt[1], c1 = g.col_cnt[0];
     const int p = c2 < c1 ? c2 : c1;
@@ -633,6 +635,7 @@ template <bool STORE_T, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(kSweepThreads, 3) k_sweep_diffuse_box(DevGrid g, int src, int tmp, int dst, float coef,
                                                                        int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[kSweepThreads / 32];
     const int n = g.ctrl->list_n;
     const int warps_total = gridDim.x * (kSweepThreads / 32);
@@ -662,6 +665,7 @@ enum { SW_DIFFUSE7 = 1, SW_BOX27 = 2 };
 template <int OP, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(kSweepThreads, 3) k_sweep_single(DevGrid g, int src, int dst, float coef, int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[kSweepThreads / 32];
     const int n = g.ctrl->list_n;
     const float *__restrict__ x = g.field[src];
@@ -913,6 +917,7 @@ template <int OP, bool CHECK, bool SUM>
 __global__ void __launch_bounds__(kSweepThreads, 4) k_sweep_single_jruns(DevGrid g, int src, int dst, float coef,
                                                                         int sum_slot)
 {
+    chained_entry();
     __shared__ double s_red[kSweepThreads / 32];
     const int c3 = g.col_cnt[2], c2 = g.col_cnt[1], c1 = g.col_cnt[0];
     const int p = c2 < c1 ? c2 : c1;
@@ -966,7 +971,7 @@ void launch_sweep_diffuse_box(const DevGrid &g, cudaStream_t s, int src, int tmp
 {
     const int ctas = sweep_ctas(lc.num_sms, 0);
     const bool sum = sum_slot >= 0;
-#define SG_SW(ST, CK, SU) k_sweep_diffuse_box<ST, CK, SU><<<ctas, kSweepThreads, 0, s>>>(g, src, tmp, dst, coef, sum_slot)
+#define SG_SW(ST, CK, SU) launch_chained(k_sweep_diffuse_box<ST, CK, SU>, ctas, kSweepThreads, 0, s, g, src, tmp, dst, coef, sum_slot)
     if (store_tmp) {
         if (check_act) { if (sum) SG_SW(true, true, true); else SG_SW(true, true, false); }
         else { if (sum) SG_SW(true, false, true); else SG_SW(true, false, false); }
@@ -982,7 +987,7 @@ void launch_sweep_columns(const DevGrid &g, cudaStream_t s, int src, int tmp, in
 {
     const int ctas = sweep_ctas(lc.num_sms, 2);
     const bool sum = sum_slot >= 0;
-#define SG_SC(ST, CK, SU) k_sweep_columns<ST, CK, SU><<<ctas, kSweepThreads, 0, s>>>(g, src, tmp, dst, coef, sum_slot)
+#define SG_SC(ST, CK, SU) launch_chained(k_sweep_columns<ST, CK, SU>, ctas, kSweepThreads, 0, s, g, src, tmp, dst, coef, sum_slot)
     if (store_tmp) {
         if (check_act) { if (sum) SG_SC(true, true, true); else SG_SC(true, true, false); }
         else { if (sum) SG_SC(true, false, true); else SG_SC(true, false, false); }
@@ -998,7 +1003,7 @@ void launch_sweep_jruns(const DevGrid &g, cudaStream_t s, int src, int tmp, int 
 {
     const int ctas = sweep_ctas(lc.num_sms, 3);
     const bool sum = sum_slot >= 0;
-#define SG_SJ(ST, CK, SU) k_sweep_jruns<ST, CK, SU><<<ctas, kSweepThreads, 0, s>>>(g, src, tmp, dst, coef, sum_slot)
+#define SG_SJ(ST, CK, SU) launch_chained(k_sweep_jruns<ST, CK, SU>, ctas, kSweepThreads, 0, s, g, src, tmp, dst, coef, sum_slot)
     if (store_tmp) {
         if (check_act) { if (sum) SG_SJ(true, true, true); else SG_SJ(true, true, false); }
         else { if (sum) SG_SJ(true, false, true); else SG_SJ(true, false, false); }
@@ -1015,7 +1020,7 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
     const bool sum = sum_slot >= 0;
     if (lc.single_runs) {
         const int ctas = sweep_ctas(lc.num_sms, 4);
-#define SG_SR(OP, CK, SU) k_sweep_single_jruns<OP, CK, SU><<<ctas, kSweepThreads, 0, s>>>(g, src, dst, coef, sum_slot)
+#define SG_SR(OP, CK, SU) launch_chained(k_sweep_single_jruns<OP, CK, SU>, ctas, kSweepThreads, 0, s, g, src, dst, coef, sum_slot)
         if (op == SW_DIFFUSE7) {
             if (check_act) { if (sum) SG_SR(SW_DIFFUSE7, true, true); else SG_SR(SW_DIFFUSE7, true, false); }
             else { if (sum) SG_SR(SW_DIFFUSE7, false, true); else SG_SR(SW_DIFFUSE7, false, false); }
@@ -1027,7 +1032,7 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
         return;
     }
     const int ctas = sweep_ctas(lc.num_sms, 1);
-#define SG_SS(OP, CK, SU) k_sweep_single<OP, CK, SU><<<ctas, kSweepThreads, 0, s>>>(g, src, dst, coef, sum_slot)
+#define SG_SS(OP, CK, SU) launch_chained(k_sweep_single<OP, CK, SU>, ctas, kSweepThreads, 0, s, g, src, dst, coef, sum_slot)
     if (op == SW_DIFFUSE7) {
         if (check_act) { if (sum) SG_SS(SW_DIFFUSE7, true, true); else SG_SS(SW_DIFFUSE7, true, false); }
         else { if (sum) SG_SS(SW_DIFFUSE7, false, true); else SG_SS(SW_DIFFUSE7, false, false); }
@@ -1051,6 +1056,7 @@ __global__ void __launch_bounds__(WARPS * 32, 16 / WARPS) k_batch_diffuse_box(co
                                                                               int n_grids, int total_tri, float coef,
                                                                               double *acc)
 {
+    chained_entry();
     __shared__ int s_off[kMaxBatch + 1];
     for (int i = threadIdx.x; i <= n_grids; i += WARPS * 32) s_off[i] = (i < n_grids) ? items[i].tri0 : total_tri;
     __syncthreads();
@@ -1091,9 +1097,9 @@ void launch_batch_diffuse_box(const BatchGrid *items, int n_grids, int total_tri
                               int num_sms, cudaStream_t s)
 {
     const int ctas = batch_ctas(num_sms, warps);
-    if (warps == 2) k_batch_diffuse_box<2><<<ctas, 64, 0, s>>>(items, n_grids, total_tri, coef, acc);
-    else if (warps == 8) k_batch_diffuse_box<8><<<ctas, 256, 0, s>>>(items, n_grids, total_tri, coef, acc);
-    else k_batch_diffuse_box<4><<<ctas, 128, 0, s>>>(items, n_grids, total_tri, coef, acc);
+    if (warps == 2) launch_chained(k_batch_diffuse_box<2>, ctas, 64, 0, s, items, n_grids, total_tri, coef, acc);
+    else if (warps == 8) launch_chained(k_batch_diffuse_box<8>, ctas, 256, 0, s, items, n_grids, total_tri, coef, acc);
+    else launch_chained(k_batch_diffuse_box<4>, ctas, 128, 0, s, items, n_grids, total_tri, coef, acc);
 }
 
 }  // namespace sg

@@ -106,6 +106,7 @@ struct sg_grid {
     int max_fuse = kMaxEwOps;          // element-wise ops per fused launch
     int flush_period = 0;              // flush once the queue holds this many ops (0: on sync / sg_flush only)
     long long known_leaves = 0;
+    unsigned long long ctrl_ver = 0;   // list version whose length host_ctrl holds (0 = none)
     sg_stats stats{};
     int latched = SG_OK;
     std::vector<void *> blocks;
@@ -1112,11 +1113,11 @@ int run_checks(sg_grid *g, sg_check_report *r, bool with_list)
 }
 
 // Flush, wait, read the control block; latch and clear device errors.
-int do_sync(sg_grid *g)
+// The end of a sync: wait for everything launched on the grid's stream, then
+// return the first latched error.
+int finish_sync(sg_grid *g)
 {
-    int rc = do_flush(g);
-    if (g->dry) return rc;
-    if (rc) return rc;
+    int rc;
     if ((rc = cuda_check(cudaMemcpyAsync(g->host_ctrl, g->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, g->stream),
                          "read control block")))
         return rc;
@@ -1140,14 +1141,23 @@ int do_sync(sg_grid *g)
                               (long long)r.nbr_bad, (long long)r.zero_leaf_bad, (long long)r.inactive_nonzero,
                               (long long)r.ctrl_bad);
     }
-    if (g->list_ver == g->mask_ver) g->known_leaves = g->host_ctrl->list_n;
+    if (g->list_ver == g->mask_ver) {
+        g->known_leaves = g->host_ctrl->list_n;
+        g->ctrl_ver = g->list_ver;
+    }
     const int out = g->latched;
     g->latched = SG_OK;
     return out;
 }
 
+int do_sync(sg_grid *g)
+{
+    const int rc = do_flush(g);
+    return rc || g->dry ? rc : finish_sync(g);
+}
+
 // Implicit sync with a current list (reads need list order).
-int sync_with_list(sg_grid *g)
+int flush_with_list(sg_grid *g)
 {
     if (g->dry) return fail(SG_ERR_INVALID, "a dry-run grid holds no data");
     int rc = do_flush(g);
@@ -1157,7 +1167,13 @@ int sync_with_list(sg_grid *g)
         if ((rc = launch_list(g, false, 0))) return rc;
         g->list_ver = g->mask_ver;
     }
-    return do_sync(g);
+    return SG_OK;
+}
+
+int sync_with_list(sg_grid *g)
+{
+    const int rc = flush_with_list(g);
+    return rc ? rc : finish_sync(g);
 }
 
 int ensure_staging(sg_grid *g)
@@ -1175,21 +1191,29 @@ int ensure_staging(sg_grid *g)
 // Packed positions of every list entry's active voxels (a current list of n
 // entries); returns their total through *total (implicit wait).  Kept while
 // the structure is unchanged: the list version keys them.
-int active_offsets(sg_grid *g, long long n, long long *total)
+int queue_active_offsets(sg_grid *g, long long n)
 {
-    // reused while no activation has touched the structure since (the list
-    // is current and the device dirty flag, read at the last sync, is clear)
-    if (g->act_ver == g->list_ver && g->act_ver != 0 && g->host_ctrl->dirty == 0) {
-        *total = g->act_total;
-        return SG_OK;
-    }
     if (!g->act_off) {
         g->act_off = (long long *)dev_alloc(g, sizeof(long long) * size_t(g->dev.cap));
         g->act_tsum = (long long *)dev_alloc(g, sizeof(long long) * size_t(g->dev.cap / kOffTile + 2));
         if (!g->act_off || !g->act_tsum) return fail(SG_ERR_OOM, "transfer offsets");
     }
     launch_active_offsets(g->dev, g->stream, n, g->act_off, g->act_tsum);
-    int rc = after_launch(g, "active offsets");
+    return after_launch(g, "active offsets");
+}
+
+// The offsets kept from an earlier transfer are those of the list as it is:
+// no activation has touched the structure since (the list is current and the
+// device dirty flag, read at the last sync, is clear).
+bool offsets_kept(const sg_grid *g) { return g->act_ver == g->list_ver && g->act_ver != 0 && g->host_ctrl->dirty == 0; }
+
+int active_offsets(sg_grid *g, long long n, long long *total)
+{
+    if (offsets_kept(g)) {
+        *total = g->act_total;
+        return SG_OK;
+    }
+    int rc = queue_active_offsets(g, n);
     if (rc) return rc;
     const int ntiles = (int)((n + kOffTile - 1) / kOffTile);
     if ((rc = cuda_check(cudaMemcpyAsync(total, g->act_tsum + ntiles, sizeof(long long), cudaMemcpyDeviceToHost,
@@ -1216,7 +1240,7 @@ int run_write_staged(sg_grid *g, const Op &o)
     int rc = ensure_list(g);
     if (rc) return rc;
     long long total = 0;
-    if (!(g->act_ver == g->list_ver && g->act_ver != 0 && g->host_ctrl->dirty == 0)) {
+    if (!offsets_kept(g)) {
         // the list length, on the host: wait for the work launched so far and
         // read the control block (no flush -- this runs inside one; device
         // errors stay latched for the next sync)
@@ -1926,30 +1950,61 @@ int sg_write_field_active(sg_grid *g, int32_t f, const float *host_vals, int64_t
     return cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
 }
 
+// One round trip to the device where the host already knows the list's length
+// (from a sync since it was generated): the gather is launched behind the
+// flushed work, and a single wait covers both and brings the control block, so
+// a batch's results of 64 grids cost 64 waits, not 128, each with the GPU busy
+// up to it (20 batched steps and the 64 reads: FIGURES_READ).
 int sg_read_field_active(sg_grid *g, int32_t f, int64_t cap, int64_t *n_active, float *host_vals)
 {
     if (!g || !valid_field(g, f) || cap < 0 || !n_active) return fail(SG_ERR_INVALID, "bad arguments");
-    int rc = sync_with_list(g);
+    int rc = flush_with_list(g);
     if (rc) return rc;
+    bool waited = false;  // everything launched so far is done and had no error
+    if (g->ctrl_ver != g->list_ver || (g->desc.flags & SG_CREATE_CHECK)) {
+        if ((rc = finish_sync(g))) return rc;
+        waited = true;
+    }
     const long long n = g->host_ctrl->list_n;
+    float *direct = nullptr;
+    if (n > 0 && !offsets_kept(g)) {
+        // the count comes back with the values when they go in place: the
+        // gather compares it with the buffer's capacity on the device
+        direct = (float *)mapped_host(host_vals, sizeof(float) * size_t(cap));
+        if (direct) {
+            if ((rc = queue_active_offsets(g, n))) return rc;
+            launch_gather_active(g->dev, g->stream, g->phys[f], direct, n, cap, g->act_off, g->act_tsum, g->lc);
+            if ((rc = after_launch(g, "gather active")) || (rc = finish_sync(g))) return rc;
+            g->act_ver = g->list_ver;
+            g->act_total = g->host_ctrl->act_total;
+            *n_active = g->act_total;
+            if (g->act_total > cap)
+                return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels", (long long)cap,
+                            g->act_total);
+            return SG_OK;
+        }
+    }
     long long total = 0;
     if (n > 0 && (rc = active_offsets(g, n, &total))) return rc;
     *n_active = total;
-    if (total > cap) return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels",
-                                 (long long)cap, total);
-    if (total == 0) return SG_OK;
-    if (!host_vals) return fail(SG_ERR_INVALID, "null buffer");
+    if (total > cap || total == 0 || !host_vals) {
+        if (!waited && (rc = finish_sync(g))) return rc;
+        if (total > cap)
+            return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels", (long long)cap,
+                        total);
+        return total == 0 ? SG_OK : fail(SG_ERR_INVALID, "null buffer");
+    }
     const size_t bytes = sizeof(float) * size_t(total);
-    float *direct = (float *)mapped_host(host_vals, bytes);
+    direct = (float *)mapped_host(host_vals, bytes);
     if (!direct && (rc = ensure_staging(g))) return rc;
-    launch_gather_active(g->dev, g->stream, g->phys[f], direct ? direct : g->dev.staging, total, g->act_off,
+    launch_gather_active(g->dev, g->stream, g->phys[f], direct ? direct : g->dev.staging, n, cap, g->act_off,
                          g->act_tsum, g->lc);
     if ((rc = after_launch(g, "gather active"))) return rc;
     if (!direct && (rc = cuda_check(cudaMemcpyAsync(host_vals, g->dev.staging, bytes, cudaMemcpyDeviceToHost,
                                                     g->stream),
                                     "copy active values")))
         return rc;
-    return cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
+    return finish_sync(g);
 }
 
 struct sg_graph {
@@ -2052,12 +2107,12 @@ int sg_read_sums(sg_grid *g, double *host, int64_t n)
 {
     if (!g || n < 0 || n > g->desc.max_sums || (n > 0 && !host)) return fail(SG_ERR_INVALID, "bad arguments");
     if (g->dry) return fail(SG_ERR_INVALID, "a dry-run grid holds no data");
-    int rc = do_sync(g);
+    int rc = do_flush(g);
     if (rc) return rc;
-    if (n == 0) return SG_OK;
-    if ((rc = cuda_check(cudaMemcpyAsync(host, g->dev.sums, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream), "copy sums")))
+    if (n > 0 &&
+        (rc = cuda_check(cudaMemcpyAsync(host, g->dev.sums, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream), "copy sums")))
         return rc;
-    return cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
+    return finish_sync(g);
 }
 
 int sg_set_stencil_variant(sg_grid *g, int32_t variant)
@@ -2277,7 +2332,10 @@ int grid_prepare_batch_finish(sg_grid *g, int src, int tmp, int dst, const int32
         g->latched = SG_OK;
         return out_rc;
     }
-    if (g->list_ver == g->mask_ver) g->known_leaves = g->host_ctrl->list_n;
+    if (g->list_ver == g->mask_ver) {
+        g->known_leaves = g->host_ctrl->list_n;
+        g->ctrl_ver = g->list_ver;
+    }
     batch_items(g, src, tmp, dst, cnt, out, n_active);
     return SG_OK;
 }

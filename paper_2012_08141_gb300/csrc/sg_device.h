@@ -49,6 +49,7 @@ struct Ctrl {
     int32_t timeout_site; // which wait gave up (0 none, 1 look-back, 2 test, 3 leaf allocation)
                           // or, with kErrCheck, 100 + the failed check
     int32_t bins_used;    // leaves holding particles in the last binned P2G
+    long long act_total;  // active voxels of the last active-offset scan
     uint32_t rr_ticket;   // run-record tiles handed out (zeroed before each region-mask launch)
     int32_t pad[1];
 };
@@ -165,13 +166,14 @@ void launch_scatter_field(const DevGrid &g, cudaStream_t s, int f, const float *
 // Active-voxel transfers: off[n] and tsum[n / kOffTile + 2] are scratch;
 // launch_active_offsets leaves the packed position of each list entry's first
 // active voxel in off[e] + tsum[e / kOffTile] and the total in
-// tsum[ceil(n / kOffTile)].  src / out hold exactly that many values.
+// tsum[ceil(n / kOffTile)] and ctrl->act_total.  src holds exactly that many
+// values; the gather writes nothing if they are more than out's cap.
 constexpr int kOffTile = 1024;
 void launch_active_offsets(const DevGrid &g, cudaStream_t s, long long n, long long *off, long long *tsum);
 void launch_scatter_active(const DevGrid &g, cudaStream_t s, int f, const float *src, long long total,
                            const long long *off, const long long *tsum, const LaunchCfg &lc);
-void launch_gather_active(const DevGrid &g, cudaStream_t s, int f, float *out, long long total, const long long *off,
-                          const long long *tsum, const LaunchCfg &lc);
+void launch_gather_active(const DevGrid &g, cudaStream_t s, int f, float *out, long long n, long long cap,
+                          const long long *off, const long long *tsum, const LaunchCfg &lc);
 
 // ---- stencil kernels (sg_stencil.cu) ----
 // check_act: eager activation-on-write check on every store (Sec. 6.3 off).

@@ -833,6 +833,7 @@ namespace sg {
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kOffTile) k_active_offsets(DevGrid g, long long n, long long *off, long long *tsum)
 {
+    chained_entry();
     __shared__ long long s_w[kOffTile / 32];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const long long e = (long long)blockIdx.x * kOffTile + threadIdx.x;
@@ -862,8 +863,9 @@ __global__ void __launch_bounds__(kOffTile) k_active_offsets(DevGrid g, long lon
 
 // Exclusive scan of the tile totals by one CTA, in place; the grand total
 // goes to tsum[ntiles].
-__global__ void __launch_bounds__(1024) k_active_offsets_top(long long *tsum, int ntiles)
+__global__ void __launch_bounds__(1024) k_active_offsets_top(DevGrid g, long long *tsum, int ntiles)
 {
+    chained_entry();
     __shared__ long long s_w[32];
     __shared__ long long s_carry;
     const int lane = lane_id(), warp = threadIdx.x >> 5;
@@ -897,14 +899,14 @@ __global__ void __launch_bounds__(1024) k_active_offsets_top(long long *tsum, in
         if (threadIdx.x == 1023) s_carry = ex + v;
         __syncthreads();
     }
-    if (threadIdx.x == 0) tsum[ntiles] = s_carry;
+    if (threadIdx.x == 0) tsum[ntiles] = g.ctrl->act_total = s_carry;
 }
 
 void launch_active_offsets(const DevGrid &g, cudaStream_t s, long long n, long long *off, long long *tsum)
 {
     const int ntiles = (int)((n + kOffTile - 1) / kOffTile);
-    k_active_offsets<<<ntiles, kOffTile, 0, s>>>(g, n, off, tsum);
-    k_active_offsets_top<<<1, 1024, 0, s>>>(tsum, ntiles);
+    launch_chained(k_active_offsets, ntiles, kOffTile, 0, s, g, n, off, tsum);
+    launch_chained(k_active_offsets_top, 1, 1024, 0, s, g, tsum, ntiles);
 }
 
 // Position in the packed array of the first active voxel at or after local
@@ -955,11 +957,12 @@ __global__ void k_scatter_active(DevGrid g, int f, const float *__restrict__ src
 // plain copy; a thread per four voxels storing its values one by one took 473
 // us, most of its stores being parts of a line.
 template <int L>
-__global__ void __launch_bounds__(256) k_gather_active(DevGrid g, int f, float *__restrict__ out, long long total,
-                                                       const long long *__restrict__ off,
-                                                       const long long *__restrict__ tsum)
+__global__ void __launch_bounds__(256) k_gather_active(DevGrid g, int f, float *__restrict__ out, int ntiles, long long cap,
+                                                       const long long *off, const long long *tsum)
 {
     chained_entry();
+    const long long total = tsum[ntiles];
+    if (total > cap) return;
     constexpr int V = L * L * L, W = V / 32, CAP = 4096, T = CAP / V;
     __shared__ float s_val[CAP];
     const long long n = g.ctrl->list_n;
@@ -1005,11 +1008,12 @@ void launch_scatter_active(const DevGrid &g, cudaStream_t s, int f, const float 
     launch_chained(k_scatter_active, lc.num_sms * 4, 256, 0, s, g, f, src, total, off, tsum);
 }
 
-void launch_gather_active(const DevGrid &g, cudaStream_t s, int f, float *out, long long total, const long long *off,
-                          const long long *tsum, const LaunchCfg &lc)
+void launch_gather_active(const DevGrid &g, cudaStream_t s, int f, float *out, long long n, long long cap,
+                          const long long *off, const long long *tsum, const LaunchCfg &lc)
 {
-    if (g.L == 8) launch_chained(k_gather_active<8>, lc.num_sms * 4, 256, 0, s, g, f, out, total, off, tsum);
-    else launch_chained(k_gather_active<4>, lc.num_sms * 4, 256, 0, s, g, f, out, total, off, tsum);
+    const int ntiles = (int)((n + kOffTile - 1) / kOffTile);
+    if (g.L == 8) launch_chained(k_gather_active<8>, lc.num_sms * 4, 256, 0, s, g, f, out, ntiles, cap, off, tsum);
+    else launch_chained(k_gather_active<4>, lc.num_sms * 4, 256, 0, s, g, f, out, ntiles, cap, off, tsum);
 }
 
 // Active voxels of the listed leaves: popcount of their mask words.

@@ -45,3 +45,35 @@ def test_packed_read_equals_masked_leaves(leaf_log2, n_leaves):
     got = g.read_field_active(0, out=pinned)
     assert np.array_equal(got, want) and (pinned[want.size:] == -1.0).all()
     g.close()
+
+
+def test_packed_read_capacity_and_versions():
+    """The count is compared with the buffer's capacity before anything is
+    written -- with offsets to compute and with kept ones, in place and staged
+    -- and a structure change between two reads is followed."""
+    import torch
+    import paper_2012_08141_gb300 as sg
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    g = _grid(3, 9, 5)
+    n = g.num_active()
+    for out in (torch.full((n,), -1.0).pin_memory().numpy(), np.full(n, -1.0, np.float32)):
+        for _ in range(2):  # offsets computed, then kept
+            with pytest.raises(sg.SgError):
+                g.read_field_active(0, out=out[:n - 1])
+            assert (out == -1.0).all()
+        assert np.array_equal(g.read_field_active(0, out=out), g.read_field(0)[_bits(g)])
+        out[:] = -1.0
+    g.activate_coords(torch.tensor([[1, 1, 1], [62, 62, 62], [33, 2, 9]], dtype=torch.int32, device="cuda"))
+    g.fill_hash(0, 6)
+    big = torch.full((n + 3,), -1.0).pin_memory().numpy()
+    got = g.read_field_active(0, out=big)
+    assert np.array_equal(got, g.read_field(0)[_bits(g)]) and got.size >= n
+    g.deactivate_all()
+    assert g.read_field_active(0, out=big).size == 0
+    g.close()
+
+
+def _bits(g):
+    _, masks = g.read_structure()
+    return np.unpackbits(masks.view(np.uint8), axis=1, bitorder="little").astype(bool)

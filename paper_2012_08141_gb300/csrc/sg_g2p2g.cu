@@ -258,12 +258,12 @@ __global__ void __launch_bounds__(256, L == 4 ? 3 : 2) k_g2p2g(DevGrid src, DevG
         int beg, end, oi = 0, oj = 0, ok = 0;
         const bool binned = bl < used;
         if (binned) {
-            const long long b = bin_list[bl];
-            beg = bin_off[8 * b];
-            end = bin_end[8 * b + 7];
-            oi = (int)(b / ((long long)R * R)) * L;
-            oj = (int)((b / R) % R) * L;
-            ok = (int)(b % R) * L;
+            const int b = bin_list[bl], bij = b / R, bi = bij / R;
+            beg = bin_off[8LL * b];
+            end = bin_end[8LL * b + 7];
+            oi = bi * L;
+            oj = (bij - bi * R) * L;
+            ok = (b - bij * R) * L;
             stage_velocities<L>(src, u0p, u1p, u2p, oi, oj, ok, s_u);
             for (int q = threadIdx.x; q < ND; q += blockDim.x) {
                 s_acc[0][q] = s_acc[1][q] = s_acc[2][q] = s_acc[3][q] = 0.f;
@@ -413,6 +413,304 @@ __global__ void __launch_bounds__(256, L == 4 ? 3 : 2) k_g2p2g(DevGrid src, DevG
     if (changed) mark_dirty(dst);
 }
 
+// ---------------------------------------------------------------------------
+// The same over 4^3 leaves: the P2G half sums by columns (see bin_columns),
+// and the next chunk's positions come into shared memory while a chunk is
+// worked on.  A bin of several chunks deals its particles to them in turn, so
+// each chunk has its share of every column whatever the order.  Particles
+// whose new base left the leaf's 4^3 cells are added to the grid by a warp each
+// (edge_node), the ones far from it, and those whose old base is more than a
+// cell outside the leaf, by their own thread.  A whole leaf of the usual ten
+// particles a cell is one chunk of 736: in chunks of 384 the columns are shorter
+// and the three of a warp less even (238 us).  2M particles: 220 us a launch at
+// two CTAs per SM without spills (the 256-thread kernel with a warp per cell:
+// 308 us; this one at three CTAs and 96 registers, spilling: 264 us).
+// ---------------------------------------------------------------------------
+struct G2P2G4Smem {
+    static constexpr int PPT = 4, CAP = 736;
+    float4 rec[4][CAP];
+    float4 buf[kBinBuf];
+    float4 u[512];                  // src velocities of nodes o - 1 .. o + 6
+    float x[3 * CAP];               // the next chunk's positions, in order
+    float words[kBinWarps][96];
+    int uslot[27];                  // src leaves o / 4 + {-1, 0, 1}^3
+    uint16_t idx[CAP + 2];
+    BinSort sort;
+};
+
+// One particle node by node: its G2P from src, its state, its P2G into dst.
+// Returns whether dst's structure changed.
+__device__ __noinline__ bool far_particle(const DevGrid &src, const DevGrid &dst, float *x, float *v, long long p,
+                                          float dt, int f_vel0, float pmass, int f_mass, int f_mom0)
+{
+    const float x0 = x[3 * p], x1 = x[3 * p + 1], x2 = x[3 * p + 2];
+    float3 u;
+    float c[9];
+    g2p_from_grid<true>(src, src.field[f_vel0], src.field[f_vel0 + 1], src.field[f_vel0 + 2], bspline(x0, src.N),
+                        bspline(x1, src.N), bspline(x2, src.N), u, c);
+    const float n0 = x0 + dt * u.x, n1 = x1 + dt * u.y, n2 = x2 + dt * u.z;
+    v[3 * p] = u.x;
+    v[3 * p + 1] = u.y;
+    v[3 * p + 2] = u.z;
+    x[3 * p] = n0;
+    x[3 * p + 1] = n1;
+    x[3 * p + 2] = n2;
+    const Spline nx = bspline(n0, dst.N), ny = bspline(n1, dst.N), nz = bspline(n2, dst.N);
+    return scatter_particle(dst, nx, ny, nz, make_rec(nx.fx, ny.fx, nz.fx, pmass, u, c, 1.f / (float)dst.N), f_mass, f_mom0);
+}
+constexpr int kFar = -2;
+
+__global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g4(const __grid_constant__ DevGrid src,
+                                                          const __grid_constant__ DevGrid dst,
+                                                          const int32_t *bin_list, const int32_t *bin_off,
+                                                          const int32_t *bin_end, const int32_t *perm,
+                                                          const int32_t *bins_used, float *x, float *v, float dt,
+                                                          int f_vel0, float pmass, int f_mass, int f_mom0)
+{
+    chained_entry();
+    using S = G2P2G4Smem;
+    constexpr int PPT = S::PPT, CAP = S::CAP;
+    extern __shared__ __align__(16) unsigned char smem[];
+    S &s = *reinterpret_cast<S *>(smem);
+    if (threadIdx.x == 0) misaligned(dst, smem, 16, 4);
+    const int N = src.N, R = src.R;
+    const float dx = 1.f / (float)N;
+    const int warp = threadIdx.x >> 5, lane = lane_id();
+    float *words = s.words[warp];
+    const float *u0p = src.field[f_vel0], *u1p = src.field[f_vel0 + 1], *u2p = src.field[f_vel0 + 2];
+    bool changed = false;
+    const int used = *bins_used;
+    // particles whose stencil missed the domain when they were binned
+    {
+        const long long key = 8LL * R * R * R;
+        const int end = bin_end[key];
+        for (int q = bin_off[key] + blockIdx.x * kBinThreads + threadIdx.x; q < end; q += gridDim.x * kBinThreads) {
+            changed |= far_particle(src, dst, x, v, perm[q], dt, f_vel0, pmass, f_mass, f_mom0);
+        }
+    }
+    int bl = blockIdx.x;
+    if (bl < used) {
+        auto leaf_of = [&](int l, int &b, int &beg, int &end) {
+            b = bin_list[l];
+            beg = bin_off[8LL * b];
+            end = bin_end[8LL * b + 7];
+        };
+        // slot of leaf o / 4 + {-1, 0, 1}^3 of src (threads 0 .. 26), -1: none
+        auto near_slot = [&](int b) {
+            const int t = threadIdx.x;
+            if (t >= 27) return -1;
+            const int bij = b / R, bi = bij / R;
+            const int li = bi + t / 9 - 1, lj = bij - bi * R + (t / 3) % 3 - 1, lk = b - bij * R + t % 3 - 1;
+            return (unsigned)li < (unsigned)R && (unsigned)lj < (unsigned)R && (unsigned)lk < (unsigned)R
+                       ? src.root[((long long)li * R + lj) * R + lk]
+                       : -1;
+        };
+        // chunk c of nch takes particles beg + c, beg + c + nch, ...
+        auto order = [&](int beg, int end, int c, int nch, int (&p)[PPT]) {
+#pragma unroll
+            for (int u = 0; u < PPT; ++u) {
+                const long long q = beg + c + (long long)((u * kBinWarps + warp) * 32 + lane) * nch;
+                p[u] = q < end ? perm[q] : -1;
+            }
+        };
+        auto request = [&](const int (&p)[PPT]) {
+#pragma unroll
+            for (int u = 0; u < PPT; ++u) {
+                const int q0 = (u * kBinWarps + warp) * 32;
+                if (__any_sync(kFull, p[u] >= 0)) {
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) {
+                        const int e = r * 32 + lane, w = e / 3, q = __shfl_sync(kFull, p[u], w);
+                        if (q >= 0) copy_word(s.x + 3 * q0 + e, x + 3LL * q + (e - 3 * w));
+                    }
+                }
+            }
+        };
+        int b, beg, end, nb = 0, nbeg = 0, nend = 0;
+        leaf_of(bl, b, beg, end);
+        int slot = near_slot(b), c = 0, nch = (end - beg + CAP - 1) / CAP;
+        int p[PPT], pn[PPT];
+        order(beg, end, 0, nch, p);
+        request(p);
+        if (bl + (int)gridDim.x < used) leaf_of(bl + gridDim.x, nb, nbeg, nend);
+        if (threadIdx.x < 65) s.sort.cnt[threadIdx.x] = 0;
+        if (threadIdx.x < 16) s.sort.all[threadIdx.x] = s.sort.bits[threadIdx.x] = 0;
+        if (threadIdx.x < 27) s.uslot[threadIdx.x] = slot;
+        __syncthreads();
+        for (;;) {
+            const bool last = c + 1 >= nch, more = !last || bl + (int)gridDim.x < used;
+            const int nnch = last ? (nend - nbeg + CAP - 1) / CAP : nch;
+            if (more) order(last ? nbeg : beg, last ? nend : end, last ? 0 : c + 1, nnch, pn);
+            if (last && more) slot = near_slot(nb);
+            const int bij = b / R, bi = bij / R;
+            const int oi = bi * 4, oj = (bij - bi * R) * 4, ok = (b - bij * R) * 4;
+            if (c == 0) {  // src's node velocities, 0 outside the domain or the leaves
+                for (int nd = threadIdx.x; nd < 512; nd += kBinThreads) {
+                    const int i = (nd >> 6) + 3, j = ((nd >> 3) & 7) + 3, k = (nd & 7) + 3;  // from o - 4
+                    const int us = s.uslot[(i >> 2) * 9 + (j >> 2) * 3 + (k >> 2)];
+                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (us >= 0) {
+                        const long long idx = ((long long)us << 6) + (((i & 3) << 4) | ((j & 3) << 2) | (k & 3));
+                        u = make_float4(u0p[idx], u1p[idx], u2p[idx], 0.f);
+                    }
+                    s.u[nd] = u;
+                }
+                __syncthreads();
+            }
+            copies_done();
+            __syncwarp();
+            // G2P, the particle's record of its new position, its cell and its
+            // rank among the cell's particles
+            int place[PPT] = {-1, -1, -1, -1};
+#pragma unroll 1
+            for (int u = 0; u < PPT; ++u) {
+                const int pu = u < 2 ? (u ? p[1] : p[0]) : (u == 2 ? p[2] : p[3]);
+                int pl = -1;
+                if (!__any_sync(kFull, pu >= 0)) break;  // warp-uniform
+                const int q = (u * kBinWarps + warp) * 32 + lane;
+                const float x0 = s.x[3 * q], x1 = s.x[3 * q + 1], x2 = s.x[3 * q + 2];
+                float xn[3] = {0.f, 0.f, 0.f}, vn[3] = {0.f, 0.f, 0.f};
+                if (pu >= 0) {
+                    const Spline ox = bspline(x0, N), oy = bspline(x1, N), oz = bspline(x2, N);
+                    const int ri = ox.base - oi + 1, rj = oy.base - oj + 1, rk = oz.base - ok + 1;
+                    pl = kFar;
+                    if ((unsigned)ri <= 5u && (unsigned)rj <= 5u && (unsigned)rk <= 5u) {
+                        float3 uu;
+                        float C[9];
+                        g2p_from_block<8, true>(s.u, ri, rj, rk, N, ox, oy, oz, uu, C);
+                        vn[0] = uu.x;
+                        vn[1] = uu.y;
+                        vn[2] = uu.z;
+                        xn[0] = x0 + dt * uu.x;
+                        xn[1] = x1 + dt * uu.y;
+                        xn[2] = x2 + dt * uu.z;
+                        const Spline nx = bspline(xn[0], N), ny = bspline(xn[1], N), nz = bspline(xn[2], N);
+                        const int ci = nx.base - oi, cj = ny.base - oj, ck = nz.base - ok;
+                        if ((unsigned)(ci + 500) <= 1000u && (unsigned)(cj + 500) <= 1000u && (unsigned)(ck + 500) <= 1000u) {
+                            const bool in = (unsigned)ci < 4u && (unsigned)cj < 4u && (unsigned)ck < 4u;
+                            const int cell = in ? (ci * 4 + cj) * 4 + ck : 64;
+                            pl = cell | atomicAdd(&s.sort.cnt[cell], 1) << 7;
+                            bin_record<true, CAP>(s.rec, q, nx.fx, ny.fx, nz.fx, uu.x, uu.y, uu.z, C, dx, !in,
+                                                  pack_cell(ci, cj, ck));
+                        }
+                    }
+                }
+                const int to = pl >= 0 ? pu : -1;  // the far ones are done below
+                __syncwarp();
+                warp_put<3>(v, to, vn, words);
+                warp_put<3>(x, to, xn, words);
+#pragma unroll
+                for (int w = 0; w < PPT; ++w)
+                    if (u == w) place[w] = pl;
+            }
+            __syncthreads();
+            if (warp == 0) bin_scan(s.sort);
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < PPT; ++u)
+                if (place[u] >= 0)
+                    s.idx[s.sort.start[place[u] & 127] + (place[u] >> 7)] = (uint16_t)((u * kBinWarps + warp) * 32 + lane);
+            __syncthreads();
+            if (more) request(pn);
+            bin_columns<true, CAP>(s.rec, s.idx, s.sort, s.buf);
+            for (int pp = s.sort.start[64] + warp; pp < s.sort.start[65] && pp < CAP; pp += kBinWarps) {
+                int i, j, k;
+                float4 t;
+                if (edge_node<true, CAP>(s.rec, s.idx[pp], oi, oj, ok, N, i, j, k, t))
+                    changed |= scatter_node(dst, i, j, k, pmass * t.x, pmass * t.y, pmass * t.z, pmass * t.w, f_mass, f_mom0);
+            }
+#pragma unroll
+            for (int u = 0; u < PPT; ++u)
+                if (place[u] == kFar) changed |= far_particle(src, dst, x, v, p[u], dt, f_vel0, pmass, f_mass, f_mom0);
+            if (last) {
+                __syncthreads();
+                // the touched nodes' sums, then the dst leaves that hold them
+                float4 t[2];
+                int where[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int nd = threadIdx.x + h * kBinThreads;
+                    where[h] = -1;
+                    if (nd >= kBinNodes) continue;
+                    int i, j, k, leaf, l;
+                    bin_node(nd, i, j, k, leaf, l);
+                    if (oi + i >= N || oj + j >= N || ok + k >= N || !node_hit(s.sort, i, j, k)) continue;
+                    t[h] = node_total(s.sort, s.buf, i, j, k);
+                    where[h] = leaf << 6 | l;
+                    atomicOr(&s.sort.bits[2 * leaf + (l >> 5)], 1u << (l & 31));
+                }
+                __syncthreads();
+                if (warp == 0) {
+                    if (lane < 8) {
+                        int ds = -1;
+                        if (s.sort.bits[2 * lane] | s.sort.bits[2 * lane + 1]) {
+                            bool fresh = false;
+                            ds = ensure_leaf(dst, ((long long)(bi + (lane >> 2)) * R + (oj >> 2) + ((lane >> 1) & 1)) * R +
+                                                      (ok >> 2) + (lane & 1), fresh);
+                            changed |= fresh;
+                        }
+                        s.sort.slot[lane] = ds;
+                    }
+                    __syncwarp();
+                    if (lane < 16) {
+                        const uint32_t want = s.sort.bits[lane];
+                        const int ds = s.sort.slot[lane >> 1];
+                        if (want && ds >= 0) {
+                            uint32_t *mw = &dst.mask[(long long)ds * 2 + (lane & 1)];
+                            if ((*(volatile uint32_t *)mw & want) != want) changed |= (atomicOr(mw, want) & want) != want;
+                        }
+                    }
+                    if (lane < 27) s.uslot[lane] = slot;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (where[h] < 0) continue;
+                    const int ds = s.sort.slot[where[h] >> 6];
+                    if (ds < 0) continue;  // pool exhausted; the error is latched
+                    const long long idx = ((long long)ds << 6) + (where[h] & 63);
+                    atomicAdd(dst.field[f_mass] + idx, pmass * t[h].x);
+                    atomicAdd(dst.field[f_mom0] + idx, pmass * t[h].y);
+                    atomicAdd(dst.field[f_mom0 + 1] + idx, pmass * t[h].z);
+                    atomicAdd(dst.field[f_mom0 + 2] + idx, pmass * t[h].w);
+                }
+                __syncthreads();
+                if (threadIdx.x < 16) s.sort.all[threadIdx.x] = s.sort.bits[threadIdx.x] = 0;
+                if (!more) break;
+                bl += gridDim.x;
+                b = nb;
+                beg = nbeg;
+                end = nend;
+                c = 0;
+                if (bl + (int)gridDim.x < used) leaf_of(bl + gridDim.x, nb, nbeg, nend);
+            } else {
+                ++c;
+                __syncthreads();  // the records are rewritten by the leaf's next chunk
+            }
+            nch = nnch;
+#pragma unroll
+            for (int u = 0; u < PPT; ++u) p[u] = pn[u];
+        }
+    }
+    if (changed) mark_dirty(dst);
+}
+
+void launch_g2p2g_4(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
+                    float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int num_sms)
+{
+    constexpr int bytes = (int)sizeof(G2P2G4Smem);
+    static std::atomic<int> resident;  // CTAs per SM; threads may race to fill it
+    int per = resident.load(std::memory_order_relaxed);
+    if (!per) {
+        cudaFuncSetAttribute(k_g2p2g4, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2p2g4, kBinThreads, bytes) != cudaSuccess || per < 1)
+            per = 1;
+        resident.store(per, std::memory_order_relaxed);
+    }
+    launch_chained(k_g2p2g4, per * num_sms, kBinThreads, bytes, s, src, dst, bins.bin_list, bins.bin_off, bins.bin_count,
+                   bins.perm, &bins.ctrl->bins_used, x, v, dt, f_vel0, pmass, f_mass, f_mom0);
+}
+
 template <int L>
 void launch_g2p2g_L(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
                     float dt, int f_vel0, float pmass, int f_mass, int f_mom0, bool pair, int num_sms)
@@ -438,7 +736,7 @@ void launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, c
 {
     if (n <= 0) return;
     const bool pair = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(v)) & 7) == 0;
-    if (dst.L == 4) launch_g2p2g_L<4>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, pair, lc.num_sms);
+    if (dst.L == 4) launch_g2p2g_4(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
     else launch_g2p2g_L<8>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, pair, lc.num_sms);
 }
 

@@ -182,43 +182,51 @@ __device__ __forceinline__ void stage_velocities_tight(const DevGrid &g, const f
 
 // G2P of one particle from a staged block of B^3 float4 node velocities (ri,
 // rj, rk: its base relative to the block's first node).  APIC as in
-// g2p_from_grid.
+// g2p_from_grid, the sums formed axis by axis: along k for each of the nine
+// (a, b), then along j, then i (240 operations for 27 nodes, not 350).
 template <int B, bool APIC>
 __device__ __forceinline__ void g2p_from_block(const float4 *s_u, int ri, int rj, int rk, int N, const Spline &sx,
                                                const Spline &sy, const Spline &sz, float3 &u, float (&c)[9])
 {
-    float ux = 0.f, uy = 0.f, uz = 0.f;
+    float U[3] = {0.f, 0.f, 0.f};
     float S[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a) {
+        const float wa = a == 0 ? sx.w[0] : (a == 1 ? sx.w[1] : sx.w[2]), ta = (float)a;
+        const float4 *plane = s_u + ((ri + a) * B + rj) * B + rk;
+        float T[3] = {0.f, 0.f, 0.f}, Tj[3] = {0.f, 0.f, 0.f}, Tk[3] = {0.f, 0.f, 0.f};
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const float wxy = sx.w[a] * sy.w[b];
+            const float4 n0 = plane[b * B], n1 = plane[b * B + 1], n2 = plane[b * B + 2];
+            const float v0[3] = {n0.x, n0.y, n0.z}, v1[3] = {n1.x, n1.y, n1.z}, v2[3] = {n2.x, n2.y, n2.z};
 #pragma unroll
-            for (int cc = 0; cc < 3; ++cc) {
-                const float4 n = s_u[((ri + a) * B + (rj + b)) * B + (rk + cc)];
-                const float w = wxy * sz.w[cc];
-                const float wv[3] = {w * n.x, w * n.y, w * n.z};
-                ux += wv[0];
-                uy += wv[1];
-                uz += wv[2];
+            for (int e = 0; e < 3; ++e) {
+                const float s1 = sz.w[1] * v1[e], s2 = sz.w[2] * v2[e];
+                const float s = fmaf(sz.w[0], v0[e], s1 + s2);
+                T[e] = fmaf(sy.w[b], s, T[e]);
                 if (APIC) {
-#pragma unroll
-                    for (int e = 0; e < 3; ++e) {
-                        if (a) S[e][0] = fmaf((float)a, wv[e], S[e][0]);
-                        if (b) S[e][1] = fmaf((float)b, wv[e], S[e][1]);
-                        if (cc) S[e][2] = fmaf((float)cc, wv[e], S[e][2]);
-                    }
+                    if (b) Tj[e] = fmaf((float)b * sy.w[b], s, Tj[e]);
+                    Tk[e] = fmaf(sy.w[b], fmaf(2.f, s2, s1), Tk[e]);
                 }
             }
         }
-    u = make_float3(ux, uy, uz);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            U[e] = fmaf(wa, T[e], U[e]);
+            if (APIC) {
+                S[e][0] = fmaf(ta * wa, T[e], S[e][0]);
+                S[e][1] = fmaf(wa, Tj[e], S[e][1]);
+                S[e][2] = fmaf(wa, Tk[e], S[e][2]);
+            }
+        }
+    }
+    u = make_float3(U[0], U[1], U[2]);
     if (APIC) {
-        const float s4 = 4.f * (float)N, fx[3] = {sx.fx, sy.fx, sz.fx}, ue[3] = {ux, uy, uz};
+        const float s4 = 4.f * (float)N, fx[3] = {sx.fx, sy.fx, sz.fx};
 #pragma unroll
         for (int e = 0; e < 3; ++e)
 #pragma unroll
-            for (int f = 0; f < 3; ++f) c[3 * e + f] = s4 * fmaf(-fx[f], ue[e], S[e][f]);
+            for (int f = 0; f < 3; ++f) c[3 * e + f] = s4 * fmaf(-fx[f], U[e], S[e][f]);
     }
 }
 
@@ -236,5 +244,246 @@ __device__ __forceinline__ BsPoly bs_poly(int t)
     return c;
 }
 __device__ __forceinline__ float bs_eval(const BsPoly &c, float f) { return fmaf(fmaf(c.a2, f, c.a1), f, c.a0); }
+
+// ---------------------------------------------------------------------------
+// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3 of a 4^3 leaf),
+// shared by the binned P2G and the fused G2P2G.  CTAs of six warps.
+//
+// The chunk's particles lie in shared memory as float4 records
+//   PIC   r0 = (f_i, f_j, z0, z2)  r1 = (v0, v1, v2, z1)
+//   APIC  r0 = (f_i, f_j, z0, z2)  r1 = (q0, q1, q2, M0)  r2 = M1..M4
+//         r3 = M5..M8,  M = dx C, q = v - M f
+// (f: spline offsets, z: the three weights along k; a unit mass: the sums are
+// scaled when they are flushed), and idx lists them by base cell, k fastest,
+// so the four cells of a column (ci, cj) are consecutive.  Nine lanes share a
+// column: lane (a, b) walks its particles and sums their contributions to the
+// nodes (ci + a, cj + b, .) in a window of three nodes along k, which moves on
+// cell by cell, so the weights along i and j and the record are read once for
+// three nodes, and three columns go side by side in a warp: the 16 columns take
+// one round of the six warps.  A finished node is stored to the lane's own
+// place in s_buf -- no atomics, which on FP32 in shared memory are compare and
+// swap loops -- and node_total adds a node's up to nine column sums.  Particles
+// outside the 4^3 cells (bucket 64, r0 = (f_i, f_j, f_k, cell)) are added to
+// the grid by a warp each (edge_node).
+// What bounds it is issue and the barriers between the phases of a bin (40 %
+// issue at 12 warps per SM).  Registers matter more than warps: at four CTAs per
+// SM (80 registers) the APIC form spills and is slower than at two.
+// ---------------------------------------------------------------------------
+constexpr int kBinThreads = 192, kBinWarps = kBinThreads / 32;
+constexpr int kBinNodes = 216;        // 6^3 nodes o .. o + 5
+constexpr int kBinBuf = 16 * 9 * 6;   // float4 [column][lane][node]
+
+struct BinSort {
+    int cnt[65];       // particles per cell (64: outside the cells); zero between chunks
+    int start[66];     // their places in idx
+    uint32_t prev[16], all[16];  // occupied cells of each column before / after this chunk
+    int slot[8];       // leaves o / 4 + {0, 1}^3
+    uint32_t bits[16]; // touched nodes of those leaves, two mask words each
+};
+
+// Exclusive scan of the cell counts (one warp), which it zeroes.
+__device__ __forceinline__ void bin_scan(BinSort &s)
+{
+    const int lane = lane_id();
+    int c[4] = {0, 0, 0, 0};
+    if (lane < 16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] = s.cnt[4 * lane + q];
+    } else if (lane == 16) {
+        c[0] = s.cnt[64];
+    }
+    const int tot = (c[0] + c[1]) + (c[2] + c[3]);
+    int run = warp_incl_scan(tot) - tot;
+    if (lane < 16) {
+        uint32_t now = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s.start[4 * lane + q] = run;
+            s.cnt[4 * lane + q] = 0;
+            run += c[q];
+            if (c[q]) now |= 1u << q;
+        }
+        const uint32_t before = s.all[lane];
+        s.prev[lane] = before;
+        s.all[lane] = before | now;
+    } else if (lane == 16) {
+        s.start[64] = run;
+        s.start[65] = run + tot;
+        s.cnt[64] = 0;
+    }
+}
+
+// idx has CAP + 1 entries at least: a particle's place is read one ahead.
+template <bool APIC, int CAP>
+__device__ __forceinline__ void bin_columns(const float4 (*rec)[CAP], const uint16_t *idx, const BinSort &s,
+                                            float4 *s_buf)
+{
+    const int lane = lane_id(), grp = lane / 9, sub = lane - 9 * grp;
+    const int col = (threadIdx.x >> 5) * 3 + grp;
+    if (grp > 2 || col > 15) return;
+    int pp = s.start[4 * col];
+    const int last = s.start[4 * col + 4];
+    if (pp >= last || last > CAP) return;
+    const int a = sub / 3, b = sub - 3 * a;
+    const BsPoly pa = bs_poly(a), pb = bs_poly(b);
+    const float ta = (float)a, tb = (float)b;
+    const bool add = s.prev[col] != 0;  // an earlier chunk stored this column's sums
+    float4 *out = s_buf + (col * 9 + sub) * 6;
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
+    auto store = [&](int k, float4 n) {
+        if (add) {
+            const float4 o = out[k];
+            n = make_float4(o.x + n.x, o.y + n.y, o.z + n.z, o.w + n.w);
+        }
+        out[k] = n;
+    };
+    int next = idx[pp];
+#pragma unroll 1
+    for (int ck = 0; ck < 4; ++ck) {
+        const int end = s.start[4 * col + ck + 1];
+        while (pp < end) {
+            const int q = next;
+            next = idx[++pp];
+            const float4 r0 = rec[0][q], r1 = rec[1][q];
+            const float w = bs_eval(pa, r0.x) * bs_eval(pb, r0.y);
+            const float w0 = w * r0.z, w1 = w * (APIC ? (1.f - r0.z) - r0.w : r1.w), w2 = w * r0.w;
+            float u0 = r1.x, u1 = r1.y, u2 = r1.z;
+            float m2 = 0.f, m5 = 0.f, m8 = 0.f;
+            if (APIC) {
+                const float4 r2 = rec[APIC ? 2 : 0][q], r3 = rec[APIC ? 3 : 0][q];
+                u0 = fmaf(r1.w, ta, fmaf(r2.x, tb, u0));
+                u1 = fmaf(r2.z, ta, fmaf(r2.w, tb, u1));
+                u2 = fmaf(r3.y, ta, fmaf(r3.z, tb, u2));
+                m2 = r2.y;
+                m5 = r3.x;
+                m8 = r3.w;
+            }
+            n0.x += w0;
+            n0.y = fmaf(w0, u0, n0.y);
+            n0.z = fmaf(w0, u1, n0.z);
+            n0.w = fmaf(w0, u2, n0.w);
+            n1.x += w1;
+            n1.y = fmaf(w1, APIC ? u0 + m2 : u0, n1.y);
+            n1.z = fmaf(w1, APIC ? u1 + m5 : u1, n1.z);
+            n1.w = fmaf(w1, APIC ? u2 + m8 : u2, n1.w);
+            n2.x += w2;
+            n2.y = fmaf(w2, APIC ? fmaf(2.f, m2, u0) : u0, n2.y);
+            n2.z = fmaf(w2, APIC ? fmaf(2.f, m5, u1) : u1, n2.z);
+            n2.w = fmaf(w2, APIC ? fmaf(2.f, m8, u2) : u2, n2.w);
+        }
+        store(ck, n0);
+        n0 = n1;
+        n1 = n2;
+        n2 = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    store(4, n0);
+    store(5, n1);
+}
+
+// Does any particle's stencil hold bin node (i, j, k) (0 .. 5 from o)?
+__device__ __forceinline__ bool node_hit(const BinSort &s, int i, int j, int k)
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            if ((unsigned)(i - a) <= 3u && (unsigned)(j - b) <= 3u) m |= s.all[(i - a) * 4 + (j - b)];
+    return (((m | (m << 1) | (m << 2)) >> k) & 1u) != 0u;
+}
+
+// Its sums over the columns that were stored.
+__device__ __forceinline__ float4 node_total(const BinSort &s, const float4 *s_buf, int i, int j, int k)
+{
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int ci = i - a, cj = j - b, col = ci * 4 + cj;
+            if ((unsigned)ci > 3u || (unsigned)cj > 3u || !s.all[col]) continue;
+            const float4 v = s_buf[(col * 9 + a * 3 + b) * 6 + k];
+            t.x += v.x;
+            t.y += v.y;
+            t.z += v.z;
+            t.w += v.w;
+        }
+    return t;
+}
+
+// Node nd of the bin: its place in the block, the leaf of BinSort::slot that
+// holds it and the local index there.
+__device__ __forceinline__ void bin_node(int nd, int &i, int &j, int &k, int &leaf, int &l)
+{
+    i = nd / 36;
+    j = nd / 6 - 6 * i;
+    k = nd - 6 * (nd / 6);
+    leaf = ((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2);
+    l = ((i & 3) << 4) | ((j & 3) << 2) | (k & 3);
+}
+
+// Cell of a particle outside the bin's cells, relative to o, in 10 bits a
+// coordinate (|.| < 512).
+__device__ __forceinline__ float pack_cell(int ri, int rj, int rk)
+{
+    return __int_as_float(((ri + 512) << 20) | ((rj + 512) << 10) | (rk + 512));
+}
+
+// A particle's record at place pos, from its spline offsets, velocity and (C
+// scaled in place) affine matrix; cell: pack_cell's word for bucket 64.
+template <bool APIC, int CAP>
+__device__ __forceinline__ void bin_record(float4 (*rec)[CAP], int pos, float fx, float fy, float fz, float v0, float v1,
+                                           float v2, float (&c)[9], float dx, bool edge, float cell)
+{
+    const float d0 = 1.5f - fz, d1 = fz - 1.0f, d2 = fz - 0.5f;
+    const float z0 = 0.5f * d0 * d0, z1 = 0.75f - d1 * d1, z2 = 0.5f * d2 * d2;
+    rec[0][pos] = make_float4(fx, fy, edge ? fz : z0, edge ? cell : z2);
+    if (!APIC) {
+        rec[1][pos] = make_float4(v0, v1, v2, z1);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) c[e] *= dx;
+        rec[1][pos] = make_float4(v0 - (c[0] * fx + c[1] * fy + c[2] * fz), v1 - (c[3] * fx + c[4] * fy + c[5] * fz),
+                                  v2 - (c[6] * fx + c[7] * fy + c[8] * fz), c[0]);
+        rec[APIC ? 2 : 0][pos] = make_float4(c[1], c[2], c[3], c[4]);
+        rec[APIC ? 3 : 0][pos] = make_float4(c[5], c[6], c[7], c[8]);
+    }
+}
+
+// Four bytes from global to shared memory, asynchronously.
+__device__ __forceinline__ void copy_word(float *dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One record outside the bin's cells, by a warp: lane (a, b, c) < 27 forms the
+// contribution of its node base + (a, b, c); false for lanes without a node in
+// the domain.  t: weight and weighted velocity.
+template <bool APIC, int CAP>
+__device__ __forceinline__ bool edge_node(const float4 (*rec)[CAP], int pp, int oi, int oj, int ok, int N, int &i, int &j,
+                                          int &k, float4 &t)
+{
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, c = lane % 3;
+    if (lane >= 27) return false;
+    const float4 r0 = rec[0][pp], r1 = rec[1][pp];
+    const int cell = __float_as_int(r0.w);
+    i = oi + (cell >> 20) - 512 + a;
+    j = oj + ((cell >> 10) & 1023) - 512 + b;
+    k = ok + (cell & 1023) - 512 + c;
+    if ((unsigned)i >= (unsigned)N || (unsigned)j >= (unsigned)N || (unsigned)k >= (unsigned)N) return false;
+    const float w = bs_eval(bs_poly(a), r0.x) * bs_eval(bs_poly(b), r0.y) * bs_eval(bs_poly(c), r0.z);
+    float u0 = r1.x, u1 = r1.y, u2 = r1.z;
+    if (APIC) {
+        const float4 r2 = rec[APIC ? 2 : 0][pp], r3 = rec[APIC ? 3 : 0][pp];
+        const float ta = (float)a, tb = (float)b, tc = (float)c;
+        u0 = fmaf(r1.w, ta, fmaf(r2.x, tb, fmaf(r2.y, tc, u0)));
+        u1 = fmaf(r2.z, ta, fmaf(r2.w, tb, fmaf(r3.x, tc, u1)));
+        u2 = fmaf(r3.y, ta, fmaf(r3.z, tb, fmaf(r3.w, tc, u2)));
+    }
+    t = make_float4(w, w * u0, w * u1, w * u2);
+    return true;
+}
 
 }  // namespace sg

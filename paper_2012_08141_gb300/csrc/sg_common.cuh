@@ -61,7 +61,8 @@ __device__ __forceinline__ void chained_entry()
 }
 
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+inline void launch_kernel(bool chained, void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s,
+                          A &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas);
@@ -72,8 +73,27 @@ inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, si
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    launch_kernel(true, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
+}
+
+// For a resident kernel whose CTAs together want more shared memory than the
+// kernel before it: an SM divides its memory between L1 and shared memory when
+// it is empty, so CTAs that come up beside the last ones of a kernel without
+// shared memory find room for one or two only, and the rest of the grid runs
+// after them (advection, six steps and the reads: 3480 us, drained 2513 us).  It is launched
+// when the kernels before it have drained; the next one may still be chained
+// to it.
+template <typename... P, typename... A>
+inline void launch_drained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    launch_kernel(false, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
 }
 
 // Mark the grid's structure as changed (an activation set a new bit or

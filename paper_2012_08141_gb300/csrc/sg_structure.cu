@@ -41,10 +41,11 @@ __device__ __forceinline__ int clamp_pred(long long v)
 // leaves take their pool slots with one atomic; 1 on small ones, where a warp
 // per cell keeps every cell in flight at once).
 // fill_mask: the (physical) fields a newly allocated leaf is zero-filled in.
-// Cell indices are 32-bit (R^3 <= 2^30).  For 8^3 leaves, word w of a cell
-// holds voxels l = 32w + lane: local i = w / 2 (the same for the whole warp),
-// j = lane / 8 + 4 (w & 1), k = lane & 7, so a lane forms its two j^2 + k^2
-// terms once per cell and each word adds the warp's i^2.
+// Cell indices are 32-bit (R^3 <= 2^30).  For 8^3 leaves a lane tests two rows
+// of a candidate's 64, eight k each, against one unsigned bound, and two
+// neighbouring lanes' bytes make a mask word: about 150 instructions a
+// candidate where a ballot per 32 voxels took 390, and issue is what bounds the
+// kernel (1024^3 band 84 -> 62 us).
 template <int L>
 __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2_, long long hi2_, int strict, int tube,
                                                         int cpw, uint32_t fill_mask)
@@ -58,10 +59,16 @@ __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2
     const unsigned RR = (unsigned)R * (unsigned)R;
     const long long nr = (long long)R * R * R;
     const int lo2 = clamp_pred(lo2_), hi2 = clamp_pred(hi2_);
+    // the predicate as one unsigned comparison: least <= D < hi2
+    const bool some = !(strict && lo2 == 2147483647);
+    const int least = strict && some ? lo2 + 1 : lo2;
+    const bool filled = (fill_mask & ((g.F < 32 ? 1u << g.F : 0u) - 1u)) != 0u;
+    const unsigned span = some && hi2 > least ? (unsigned)hi2 - (unsigned)least : 0u;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long c0 = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * cpw; c0 < nr; c0 += warps * cpw) {
         // lane q < cpw tests cell c0 + q: can its bounding box meet the band?
         bool cand = false;
+        uint32_t cell = 0;  // its (i, j, k), 10 bits each (R <= 1024)
         const long long bq = c0 + lane;
         if (lane < cpw && bq < nr) {
             const unsigned b = (unsigned)bq, bi = b / RR, rem = b - bi * RR, bj = rem / (unsigned)R,
@@ -72,44 +79,43 @@ __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2
             if (!tube) axis_range((int)bk * L, L, N, dmin, dmax);
             const bool lo_possible = strict ? (dmax > lo2) : (dmax >= lo2);
             cand = lo_possible && dmin < hi2;
+            cell = (bi << 20) | (bj << 10) | bk;
         }
-        // the mask words of every candidate, one ballot per 32 voxels
+        // the mask words of every candidate
         bool any_bits = false;  // lane q: cell c0 + q has an active voxel
         unsigned todo = __ballot_sync(kFull, cand);
         while (todo) {
             const int q = __ffs(todo) - 1;
             todo &= todo - 1;
-            const unsigned b = (unsigned)(c0 + q), bi = b / RR, rem = b - bi * RR, bj = rem / (unsigned)R,
-                           bk = rem - bj * (unsigned)R;
-            uint32_t bits = 0;
+            const uint32_t cq = __shfl_sync(kFull, cell, q);
+            const int bi = (int)(cq >> 20), bj = (int)((cq >> 10) & 1023u), bk = (int)(cq & 1023u);
+            uint32_t bits = 0;  // word w in lane 2w (8^3) or w (4^3)
             if (L == 8) {
-                const int d = 2 * ((int)bk * 8 + (lane & 7)) + 1 - N;
-                const int dd = tube ? 0 : d * d;
-                const int cA = 2 * ((int)bj * 8 + (lane >> 3)) + 1 - N, cB = cA + 8;
-                const int e0 = cA * cA + dd, e1 = cB * cB + dd;
+                // rows 2 lane and 2 lane + 1 of the leaf (the same i, j and j + 1)
+                const int a = 2 * (bi * 8 + (lane >> 2)) + 1 - N, c = 2 * (bj * 8 + 2 * (lane & 3)) + 1 - N;
+                const int r0 = a * a + c * c - least, r1 = r0 + 4 * c + 4;  // (c + 2)^2 = c^2 + 4 c + 4
+                const int d0 = 2 * bk * 8 + 1 - N;
 #pragma unroll
-                for (int w = 0; w < W; ++w) {
-                    const int a = 2 * ((int)bi * 8 + (w >> 1)) + 1 - N;
-                    const int D = a * a + ((w & 1) ? e1 : e0);
-                    const bool on = (strict ? (lo2 < D) : (lo2 <= D)) && (D < hi2);
-                    const unsigned word = __ballot_sync(kFull, on);
-                    if (lane == w) bits = word;
+                for (int k = 0; k < 8; ++k) {
+                    const int d = d0 + 2 * k, dd = tube ? 0 : d * d;
+                    if ((unsigned)(r0 + dd) < span) bits |= 1u << k;
+                    if ((unsigned)(r1 + dd) < span) bits |= 256u << k;
                 }
+                bits |= __shfl_down_sync(kFull, bits, 1) << 16;  // used in the even lanes
+                if (!(lane & 1)) s_bits[warp][q][lane >> 1] = bits;
             } else {
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
                     const int l = w * 32 + lane;
                     const int li = l >> (2 * LG2), lj = (l >> LG2) & (L - 1), lk = l & (L - 1);
-                    const int a = 2 * ((int)bi * L + li) + 1 - N;
-                    const int c = 2 * ((int)bj * L + lj) + 1 - N;
-                    const int d = 2 * ((int)bk * L + lk) + 1 - N;
-                    const int D = a * a + c * c + (tube ? 0 : d * d);
-                    const bool on = (strict ? (lo2 < D) : (lo2 <= D)) && (D < hi2);
-                    const unsigned word = __ballot_sync(kFull, on);
+                    const int a = 2 * (bi * L + li) + 1 - N;
+                    const int c = 2 * (bj * L + lj) + 1 - N;
+                    const int d = 2 * (bk * L + lk) + 1 - N;
+                    const unsigned word = __ballot_sync(kFull, (unsigned)(a * a + c * c + (tube ? 0 : d * d) - least) < span);
                     if (lane == w) bits = word;
                 }
+                if (lane < W) s_bits[warp][q][lane] = bits;
             }
-            if (lane < W) s_bits[warp][q][lane] = bits;
             const bool nz = __any_sync(kFull, bits != 0u);
             if (lane == q) any_bits = nz;
         }
@@ -147,14 +153,13 @@ __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2
             constexpr int V = L * L * L;
             if (fq) {
                 const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int f = 0; f < g.F; ++f) {
-                    if (!((fill_mask >> f) & 1u)) continue;
-                    float4 *p = reinterpret_cast<float4 *>(g.field[f] + (long long)sq * V);
-                    for (int qq = lane; qq < V / 4; qq += 32) p[qq] = z;
-                }
+                if (filled)
+                    for (int f = 0; f < g.F; ++f) {
+                        if (!((fill_mask >> f) & 1u)) continue;
+                        float4 *p = reinterpret_cast<float4 *>(g.field[f] + (long long)sq * V);
+                        for (int qq = lane; qq < V / 4; qq += 32) p[qq] = z;
+                    }
                 if (lane < W) g.mask[(long long)sq * W + lane] = s_bits[warp][q][lane];
-                __syncwarp();
-                if (lane == 0) g.root[c0 + q] = sq;
                 changed = true;
             } else if (lane < W) {
                 uint32_t *m = &g.mask[(long long)sq * W + lane];
@@ -165,6 +170,7 @@ __global__ void __launch_bounds__(256) k_activate_shell(DevGrid g, long long lo2
                 }
             }
         }
+        if (fresh) g.root[c0 + lane] = slot;
         if (__any_sync(kFull, changed) && lane == 0) mark_dirty(g);
         __syncwarp();  // s_bits is reused by the next chunk
     }
@@ -693,7 +699,7 @@ void launch_region_masks(const DevGrid &g, cudaStream_t s, const LaunchCfg &lc, 
                          unsigned long long call)
 {
     if (group_axis != kGroupNone) cudaMemsetAsync(&g.ctrl->rr_ticket, 0, sizeof(uint32_t), s);
-    launch_chained(k_region_masks, lc.num_sms * 4, 256, 0, s, g, group_axis, call);
+    launch_chained(k_region_masks, lc.num_sms * 8, 256, 0, s, g, group_axis, call);
 }
 
 // ---------------------------------------------------------------------------

@@ -875,19 +875,19 @@ void drop_dead_sums(sg_grid *g)
     g->queue.swap(kept);
 }
 
-// Binned-P2G scratch: bin counts and offsets over the root cells, the count
-// scan's tile sums, and a particle order array of at least n entries.
+// Binned-P2G scratch: counts and offsets of the bins, reach classes of the root
+// cells, the count scan's tile sums, and a particle order array of at least n entries.
 int ensure_p2g_scratch(sg_grid *g, long long n)
 {
     if (g->dry) return SG_OK;
-    const long long nbins = (long long)g->dev.R * g->dev.R * g->dev.R;
-    const long long nkeys = p2g_num_keys(g->dev.R);
+    const long long nbins = p2g_bins(g->dev.R, g->dev.lg2), words = p2g_words(nbins);
     if (!g->dev.bin_count) {
-        g->dev.bin_count = (int32_t *)dev_alloc(g, sizeof(int32_t) * nkeys);
-        g->dev.bin_off = (int32_t *)dev_alloc(g, sizeof(int32_t) * nkeys);
-        g->dev.tile_sum = (int32_t *)dev_alloc(g, sizeof(int32_t) * (nkeys / 1024 + 2));
-        g->dev.bin_list = (int32_t *)dev_alloc(g, sizeof(int32_t) * (nbins + 1));
-        if (!g->dev.bin_count || !g->dev.bin_off || !g->dev.tile_sum || !g->dev.bin_list)
+        g->dev.bin_count = (int32_t *)dev_alloc(g, sizeof(int32_t) * words);
+        g->dev.bin_reach = (uint32_t *)dev_alloc(g, sizeof(uint32_t) * p2g_words(p2g_bins(g->dev.R, 2)));
+        g->dev.bin_off = (int32_t *)dev_alloc(g, sizeof(int32_t) * words);
+        g->dev.tile_sum = (int32_t *)dev_alloc(g, sizeof(int32_t) * (words / kBinTile));
+        g->dev.bin_list = (int32_t *)dev_alloc(g, sizeof(int32_t) * nbins);
+        if (!g->dev.bin_count || !g->dev.bin_reach || !g->dev.bin_off || !g->dev.tile_sum || !g->dev.bin_list)
             return fail(SG_ERR_OOM, "p2g bins");
     }
     if (n > g->perm_cap) {
@@ -895,7 +895,7 @@ int ensure_p2g_scratch(sg_grid *g, long long n)
         const long long cap = std::max(n, g->perm_cap * 2);
         g->dev.perm = (int32_t *)dev_alloc(g, sizeof(int32_t) * cap);
         g->dev.perm_alt = (int32_t *)dev_alloc(g, sizeof(int32_t) * cap);
-        g->dev.perm_key = (long long *)dev_alloc(g, sizeof(long long) * cap);
+        g->dev.perm_key = (int32_t *)dev_alloc(g, sizeof(int32_t) * cap);
         if (!g->dev.perm || !g->dev.perm_alt || !g->dev.perm_key)
             return fail(SG_ERR_OOM, "p2g order of %lld particles", cap);
         g->perm_cap = cap;
@@ -992,7 +992,7 @@ int do_flush(sg_grid *g)
                 if (!(rc = ensure_p2g_scratch(g, o.n))) {
                     // the same particles binned before: rebin from their last order
                     const bool rebin = g->p2g_x == o.p0 && g->p2g_n == o.n;
-                    const int k = g->dry ? 7
+                    const int k = g->dry ? p2g_launches(g->dev)
                                          : launch_p2g_binned(g->dev, g->stream, (const float *)o.p0,
                                                              (const float *)o.p1, (const float *)o.p3, o.n, o.f0,
                                                              o.i0, o.i1, rebin, g->lc);

@@ -71,14 +71,18 @@ struct DevGrid {
     Ctrl *ctrl;
     float *staging;      // n * L^3 floats for host reads/writes
     uint32_t *staging_u; // aliases staging for mask gathers
-    // binned P2G scratch (allocated at the first P2G): per-key counts/cursors
-    // and offsets, tile sums of the count scan, particle order
+    // binned P2G scratch (allocated at the first P2G): a word per bin (4^3
+    // block of the domain), one for the particles whose stencil misses the
+    // domain, and padding to whole tiles -- counts, then insertion cursors (at
+    // the end the ends of the bins' ranges), and starts; the reach classes
+    // seen of each root cell; tile sums of the counts
     int32_t *bin_count;
+    uint32_t *bin_reach;
     int32_t *bin_off;
     int32_t *tile_sum;
     int32_t *perm;
     int32_t *perm_alt;  // the next binning's order, built from the last one (then swapped)
-    long long *perm_key;  // each particle's key, stored by the count pass for the order pass
+    int32_t *perm_key;    // each particle's bin, stored by the count pass for the order pass
     int32_t *bin_list;  // the leaves holding particles, in no particular order
     // grouped sweeps of the fused step: list entry of each slot (written by
     // the list generation), the records of runs of adjacent leaves (along i
@@ -263,10 +267,15 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
 
 // ---- particle kernels (sg_particle.cu) ----
 // Binned P2G (count, allocate, scan, order, accumulate per bin); returns the
-// number of kernels launched.  Needs bin_count/bin_off (p2g_num_keys each),
-// tile_sum, perm and bin_list (R^3).  Keys: 8 reach classes per leaf plus one
-// for particles whose stencil misses the domain.
-constexpr long long p2g_num_keys(int R) { return 8LL * R * R * R + 1; }
+// number of kernels launched.  A bin is a 4^3 block of base nodes: a leaf, or
+// an eighth of an 8^3 leaf (numbered by leaf, then by octant).  Needs
+// bin_count / bin_off (p2g_words(p2g_bins) each), bin_reach
+// (p2g_words(R^3)), tile_sum (a word per kBinTile bin words), perm and
+// bin_list (p2g_bins).
+constexpr int kBinTile = 1024;
+__host__ __device__ constexpr long long p2g_bins(int R, int lg2) { return (long long)R * R * R << (3 * (lg2 - 2)); }
+__host__ __device__ constexpr long long p2g_words(long long bins) { return (bins + kBinTile) / kBinTile * kBinTile; }
+int p2g_launches(const DevGrid &g);  // kernels of one binned P2G
 // C: NULL for PIC, else the APIC matrices (n x 9 FP32, row-major).
 // rebin: the particle order of the last binning of the same particles is
 // valid in g.perm; the new order is built from it in g.perm_alt (fewer

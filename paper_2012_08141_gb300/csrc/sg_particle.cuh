@@ -130,54 +130,48 @@ __device__ __forceinline__ void warp_put(float *__restrict__ a, int p, const flo
     }
 }
 
-// Stage the velocities of the (L+4)^3 nodes from o - 2 to o + L + 1 of a
-// leaf with origin o as one float4 (u0, u1, u2, 0) per node: 0 outside the
-// domain or the allocated leaves.
+// 4^3 blocks, the bins of the particle kernels: a 4^3 leaf, or an octant of an
+// 8^3 one.  A bin's number is its leaf's times 8 plus the octant; a block's
+// slot is its leaf's slot numbered the same way (an int: 2^28 leaves of 8^3
+// floats are more than the device holds).
 template <int L>
-__device__ __forceinline__ void stage_velocities(const DevGrid &g, const float *__restrict__ f0,
-                                                 const float *__restrict__ f1, const float *__restrict__ f2, int oi,
-                                                 int oj, int ok, float4 *s_u)
+__device__ __forceinline__ void bin_block(int b, int R, int &bi, int &bj, int &bk)
 {
-    constexpr int LG2 = (L == 8) ? 3 : 2, B = L + 4, NB = B * B * B;
-    const int N = g.N, R = g.R;
-    for (int nd = threadIdx.x; nd < NB; nd += blockDim.x) {
-        const int i = oi - 2 + nd / (B * B), j = oj - 2 + (nd / B) % B, k = ok - 2 + nd % B;
-        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-        if ((unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N && (unsigned)k < (unsigned)N) {
-            const int slot = __ldg(g.root + ((long long)(i >> LG2) * R + (j >> LG2)) * R + (k >> LG2));
-            if (slot >= 0) {
-                const long long idx =
-                    ((long long)slot << (3 * LG2)) + (((i & (L - 1)) << LG2) + (j & (L - 1))) * L + (k & (L - 1));
-                u = make_float4(__ldg(f0 + idx), __ldg(f1 + idx), __ldg(f2 + idx), 0.f);
-            }
-        }
-        s_u[nd] = u;
+    const int leaf = L == 8 ? b >> 3 : b, lij = leaf / R;
+    bi = lij / R;
+    bj = lij - bi * R;
+    bk = leaf - lij * R;
+    if (L == 8) {
+        bi = 2 * bi + (b >> 2 & 1);
+        bj = 2 * bj + (b >> 1 & 1);
+        bk = 2 * bk + (b & 1);
     }
 }
-
-// The (L+2)^3 nodes from o to o + L + 1 only: every node the stencils of
-// particles with base in the leaf reach (no margin for particles that moved
-// since they were binned).
 template <int L>
-__device__ __forceinline__ void stage_velocities_tight(const DevGrid &g, const float *__restrict__ f0,
-                                                       const float *__restrict__ f1, const float *__restrict__ f2,
-                                                       int oi, int oj, int ok, float4 *s_u)
+__device__ __forceinline__ long long block_leaf(int R, int bi, int bj, int bk)
 {
-    constexpr int LG2 = (L == 8) ? 3 : 2, B = L + 2, NB = B * B * B;
-    const int N = g.N, R = g.R;
-    for (int nd = threadIdx.x; nd < NB; nd += blockDim.x) {
-        const int i = oi + nd / (B * B), j = oj + (nd / B) % B, k = ok + nd % B;
-        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < N && j < N && k < N) {
-            const int slot = __ldg(g.root + ((long long)(i >> LG2) * R + (j >> LG2)) * R + (k >> LG2));
-            if (slot >= 0) {
-                const long long idx =
-                    ((long long)slot << (3 * LG2)) + (((i & (L - 1)) << LG2) + (j & (L - 1))) * L + (k & (L - 1));
-                u = make_float4(__ldg(f0 + idx), __ldg(f1 + idx), __ldg(f2 + idx), 0.f);
-            }
-        }
-        s_u[nd] = u;
-    }
+    constexpr int S = L == 8 ? 1 : 0;
+    return ((long long)(bi >> S) * R + (bj >> S)) * R + (bk >> S);
+}
+template <int L>
+__device__ __forceinline__ int block_of_leaf(int slot, int bi, int bj, int bk)
+{
+    return L == 4 || slot < 0 ? slot : slot * 8 + ((bi & 1) << 2 | (bj & 1) << 1 | (bk & 1));
+}
+// Slot of block (bi, bj, bk), negative if there is none or it lies outside the domain.
+template <int L>
+__device__ __forceinline__ int block_slot(const int32_t *root, int R, int bi, int bj, int bk)
+{
+    constexpr int S = L == 8 ? 1 : 0;
+    if ((unsigned)bi >= (unsigned)(R << S) || (unsigned)bj >= (unsigned)(R << S) || (unsigned)bk >= (unsigned)(R << S)) return -1;
+    return block_of_leaf<L>(root[block_leaf<L>(R, bi, bj, bk)], bi, bj, bk);
+}
+// Voxel (i, j, k) (0 .. 3) of a block: its index in the fields.
+template <int L>
+__device__ __forceinline__ long long block_voxel(int bs, int i, int j, int k)
+{
+    if (L == 4) return (long long)bs << 6 | (i << 4 | j << 2 | k);
+    return (long long)(bs >> 3) << 9 | ((bs & 4) << 6 | i << 6 | (bs & 2) << 4 | j << 3 | (bs & 1) << 2 | k);
 }
 
 // G2P of one particle from a staged block of B^3 float4 node velocities (ri,
@@ -246,8 +240,7 @@ __device__ __forceinline__ BsPoly bs_poly(int t)
 __device__ __forceinline__ float bs_eval(const BsPoly &c, float f) { return fmaf(fmaf(c.a2, f, c.a1), f, c.a0); }
 
 // ---------------------------------------------------------------------------
-// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3 of a 4^3 leaf),
-// shared by the binned P2G and the fused G2P2G.  CTAs of six warps.
+// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3), shared by the binned P2G and the fused G2P2G.  CTAs of six warps.
 //
 // The chunk's particles lie in shared memory as float4 records
 //   PIC   r0 = (f_i, f_j, z0, z2)  r1 = (v0, v1, v2, z1)
@@ -277,8 +270,8 @@ struct BinSort {
     int cnt[65];       // particles per cell (64: outside the cells); zero between chunks
     int start[66];     // their places in idx
     uint32_t prev[16], all[16];  // occupied cells of each column before / after this chunk
-    int slot[8];       // leaves o / 4 + {0, 1}^3
-    uint32_t bits[16]; // touched nodes of those leaves, two mask words each
+    int slot[8];       // blocks o / 4 + {0, 1}^3
+    uint32_t bits[16]; // touched nodes of those blocks, i, j, k in order
 };
 
 // Exclusive scan of the cell counts (one warp), which it zeroes.
@@ -411,15 +404,41 @@ __device__ __forceinline__ float4 node_total(const BinSort &s, const float4 *s_b
     return t;
 }
 
-// Node nd of the bin: its place in the block, the leaf of BinSort::slot that
+// Node nd of the bin: its place among the 6^3, the block of BinSort::slot that
 // holds it and the local index there.
-__device__ __forceinline__ void bin_node(int nd, int &i, int &j, int &k, int &leaf, int &l)
+__device__ __forceinline__ void bin_node(int nd, int &i, int &j, int &k, int &blk, int &l)
 {
     i = nd / 36;
     j = nd / 6 - 6 * i;
     k = nd - 6 * (nd / 6);
-    leaf = ((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2);
+    blk = ((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2);
     l = ((i & 3) << 4) | ((j & 3) << 2) | (k & 3);
+}
+
+// Set the touched nodes' bits in their leaves' masks (one warp; a lane per mask
+// word: two of a 4^3 leaf, four of a block in an 8^3 one).  Returns whether
+// this lane set a new one.
+template <int L>
+__device__ __forceinline__ bool set_touched(const DevGrid &g, const BinSort &s)
+{
+    const int lane = lane_id();
+    int bs;
+    uint32_t want;
+    long long word;
+    if (L == 4) {
+        if (lane >= 16) return false;
+        bs = s.slot[lane >> 1];
+        want = s.bits[lane];
+        word = (long long)bs * 2 + (lane & 1);
+    } else {
+        bs = s.slot[lane >> 2];
+        const uint32_t h = s.bits[lane >> 1] >> ((lane & 1) << 4);  // the plane's 16 bits, k fastest
+        want = ((h & 0xfu) | (h & 0xf0u) << 4 | (h & 0xf00u) << 8 | (h & 0xf000u) << 12) << ((bs & 1) << 2);
+        word = (long long)(bs >> 3) * 16 + ((bs & 4) + (lane & 3)) * 2 + (bs >> 1 & 1);
+    }
+    if (!want || bs < 0) return false;
+    uint32_t *mw = g.mask + word;
+    return (*(volatile uint32_t *)mw & want) != want && (atomicOr(mw, want) & want) != want;
 }
 
 // Cell of a particle outside the bin's cells, relative to o, in 10 bits a

@@ -231,83 +231,15 @@ void launch_mark_coords(const DevGrid &g, cudaStream_t s, const int32_t *xyz, lo
     k_mark_coords<<<(unsigned)blocks, 256, 0, s>>>(g, xyz, n);
 }
 
-// fill_mask: the (physical) fields a newly allocated leaf is zero-filled in.
-// A CTA takes 128 consecutive root cells: its first four warps give slots to
-// the needed null ones (one pool atomic per warp) and list them, then all of
-// its threads zero the listed leaves together.  Needed cells come in runs along
-// k, so a warp that allocated and filled its own 32 cells' leaves one after the
-// other was the launch's long pole (2M particles over 4,076 leaves 10.1 -> 4.8 us,
-// 100k particles in a 25^3 root 11.8 -> 3.7 us).
-constexpr int kAllocCells = 128;
 __global__ void __launch_bounds__(256) k_alloc_needed(DevGrid g, uint32_t fill_mask)
 {
     chained_entry();
-    __shared__ int s_slot[kAllocCells];
-    __shared__ int s_n;
-    const long long nr = (long long)g.R * g.R * g.R;
-    const int V4 = (g.L * g.L * g.L) >> 2, W = g.W;
-    bool any_alloc = false;
-    for (long long base = (long long)blockIdx.x * kAllocCells; base < nr; base += (long long)gridDim.x * kAllocCells) {
-        const long long b = base + threadIdx.x;
-        bool need = false;
-        if (threadIdx.x < kAllocCells && b < nr && g.need[b]) {
-            g.need[b] = 0;
-            need = true;
-        }
-        if (!__syncthreads_or(need)) continue;
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        int slot = -1;
-        if (threadIdx.x < kAllocCells) {
-            const bool want = need && g.root[b] < 0;
-            const unsigned m = __ballot_sync(kFull, want);
-            if (m) {
-                const int leader = __ffs(m) - 1;
-                int first = 0, at = 0;
-                if (lane_id() == leader) {
-                    first = atomicAdd(&g.ctrl->pool_count, __popc(m));
-                    at = atomicAdd(&s_n, __popc(m));
-                }
-                first = __shfl_sync(kFull, first, leader);
-                at = __shfl_sync(kFull, at, leader);
-                if (want) {
-                    const int rank = __popc(m & lanemask_lt());
-                    if (first + rank < g.cap) slot = first + rank;
-                    else raise_error(g, kErrPool);
-                    s_slot[at + rank] = slot;
-                }
-            }
-        }
-        __syncthreads();
-        const int n = s_n;
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int f = 0; f < g.F; ++f) {
-            if (!((fill_mask >> f) & 1u)) continue;
-            float4 *p = reinterpret_cast<float4 *>(g.field[f]);
-            for (int q = threadIdx.x; q < n * V4; q += 256) {
-                const int s = s_slot[q / V4];
-                if (s >= 0) p[(long long)s * V4 + (q & (V4 - 1))] = z;
-            }
-        }
-        for (int q = threadIdx.x; q < n * W; q += 256) {
-            const int s = s_slot[q / W];
-            if (s >= 0) g.mask[(long long)s * W + (q & (W - 1))] = 0u;
-        }
-        if (slot >= 0) {
-            g.root[b] = slot;
-            any_alloc = true;
-        }
-        __syncthreads();  // s_slot is refilled for the next cells
-    }
-    if (any_alloc) mark_dirty(g);
+    alloc_needed(g, fill_mask, blockIdx.x, gridDim.x);
 }
 
 void launch_alloc_needed(const DevGrid &g, cudaStream_t s, uint32_t fill_mask)
 {
-    const long long nr = (long long)g.R * g.R * g.R;
-    long long blocks = (nr + kAllocCells - 1) / kAllocCells;
-    if (blocks > 4096) blocks = 4096;
-    launch_chained(k_alloc_needed, (unsigned)blocks, 256, 0, s, g, fill_mask);
+    launch_chained(k_alloc_needed, alloc_needed_ctas(g), 256, 0, s, g, fill_mask);
 }
 
 __global__ void k_setbits_coords(DevGrid g, const int32_t *__restrict__ xyz, long long n)

@@ -1355,26 +1355,26 @@ int grid_create(const sg_desc *desc, void *cuda_stream, sg_grid **out, bool init
     }
     // initial state: all pointers null, empty pool and list, structure dirty
     cudaStream_t s = g->stream;
-    rc = cuda_check(cudaMemsetAsync(d.root, 0xff, sizeof(int32_t) * nr, s), "init root");
-    if (!rc) rc = cuda_check(cudaMemsetAsync(d.need, 0, (size_t)nr, s), "init need");
-    if (!rc) rc = cuda_check(cudaMemsetAsync(d.tile_status, 0, sizeof(unsigned long long) * g->num_tiles, s), "init status");
-    if (!rc)
-        rc = cuda_check(cudaMemsetAsync(d.rr_status, 0, sizeof(unsigned long long) * 3 * (d.cap / 256 + 1), s),
-                        "init run-record status");
-    if (!rc) rc = cuda_check(cudaMemsetAsync(d.sums, 0, sizeof(double) * std::max(1, desc->max_sums), s), "init sums");
+    InitSpans sp{};
+    int ns = 0;
+    auto span = [&](void *p, size_t bytes, int byte) { sp.span[ns++] = {p, (long long)bytes, byte ? 0xffffffffu : 0u}; };
+    span(d.root, sizeof(int32_t) * nr, 0xff);
+    span(d.need, (size_t)nr, 0);
+    span(d.tile_status, sizeof(unsigned long long) * g->num_tiles, 0);
+    span(d.rr_status, sizeof(unsigned long long) * 3 * (d.cap / 256 + 1), 0);
+    span(d.sums, sizeof(double) * std::max(1, desc->max_sums), 0);
     // the zero leaf (slot cap): never allocated, read in place of null neighbours
-    if (!rc) rc = cuda_check(cudaMemsetAsync(d.mask + d.W * d.cap, 0, sizeof(uint32_t) * d.W, s), "init zero leaf");
-    for (int f = 0; f < d.F && !rc; ++f)
-        rc = cuda_check(cudaMemsetAsync(d.field[f] + V * d.cap, 0, sizeof(float) * V, s), "init zero leaf");
-    if (!rc) {
-        Ctrl c{};
-        c.dirty = 1;
-        std::memcpy(g->host_ctrl, &c, sizeof c);
-        rc = cuda_check(cudaMemcpyAsync(d.ctrl, g->host_ctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, s), "init ctrl");
-    }
+    span(d.mask + d.W * d.cap, sizeof(uint32_t) * d.W, 0);
+    for (int f = 0; f < d.F; ++f) span(d.field[f] + V * d.cap, sizeof(float) * V, 0);
+    sp.n = ns;
+    Ctrl c{};
+    c.dirty = 1;
+    std::memcpy(g->host_ctrl, &c, sizeof c);
+    launch_init_grid(s, sp, d.ctrl, c, g->lc);
+    rc = cuda_check(cudaPeekAtLastError(), "grid initialisation");
     if (!rc && init_sync) rc = cuda_check(cudaStreamSynchronize(s), "init sync");
     if (rc) {
-        cudaStreamSynchronize(s);  // the queued initialisation still reads host_ctrl
+        cudaStreamSynchronize(s);  // the queued initialisation still writes the blocks
         cudaFreeHost(g->host_ctrl);
         dev_free_all(g);
         delete g;

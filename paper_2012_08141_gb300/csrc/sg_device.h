@@ -254,6 +254,17 @@ int grid_prepare_batch_finish(sg_grid *g, int src, int tmp, int dst, const int32
 int grid_create(const sg_desc *desc, void *cuda_stream, sg_grid **out, bool init_sync);
 int grid_num_sms(const sg_grid *g);
 
+// ---- initial state of a new grid (sg_structure.cu) ----
+struct InitSpans {
+    struct Span {
+        void *p;
+        long long bytes;
+        uint32_t word;  // 0 or all ones
+    } span[6 + kMaxFields];
+    int n;
+};
+void launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc);
+
 // ---- device-side fill with the counter-based generator (sg_structure.cu) ----
 void launch_fill_hash(const DevGrid &g, cudaStream_t s, int f, unsigned long long seed, const LaunchCfg &lc);
 

@@ -656,6 +656,34 @@ __device__ __forceinline__ float hash24(unsigned long long z)
     return fmaf(b, 0x1p-24f, fmaf(a, 0x1p-16f, -128.5f));
 }
 
+// The initial state of a new grid in one launch: the arrays of a small grid
+// are far smaller than the time that nine memsets and a copy take one after the
+// other, and every admission of a served job waits for them (24 served jobs
+// 9.76 -> 9.62 ms).  16 bytes a thread where the span allows it.
+__global__ void __launch_bounds__(256) k_init_grid(const __grid_constant__ InitSpans in, Ctrl *ctrl,
+                                                   const __grid_constant__ Ctrl state)
+{
+    chained_entry();
+    const long long t = blockIdx.x * 256LL + threadIdx.x, nt = gridDim.x * 256LL;
+    if (t == 0) *ctrl = state;
+    for (int q = 0; q < in.n; ++q) {
+        uint8_t *p = (uint8_t *)in.span[q].p;
+        const long long bytes = in.span[q].bytes;
+        const uint32_t w = in.span[q].word;
+        const long long n16 = ((uintptr_t)p & 15) == 0 ? bytes >> 4 : 0;
+        for (long long e = t; e < n16; e += nt) reinterpret_cast<uint4 *>(p)[e] = make_uint4(w, w, w, w);
+        for (long long e = (n16 << 4) + t; e < bytes; e += nt) p[e] = (uint8_t)w;
+    }
+}
+
+void launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc)
+{
+    long long bytes = 0;
+    for (int q = 0; q < spans.n; ++q) bytes += spans.span[q].bytes;
+    const long long ctas = (bytes + 4095) / 4096, most = lc.num_sms * 8LL;
+    launch_chained(k_init_grid, ctas < most ? ctas : most, 256, 0, s, spans, ctrl, state);
+}
+
 // A group of G = min(32, L^3 / 4) threads fills one leaf, four k-adjacent
 // voxels (one float4 store) per thread and iteration: the leaf's slot, its
 // two root divisions and the row's linear index are worked out once per leaf

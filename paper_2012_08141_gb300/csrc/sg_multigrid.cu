@@ -112,42 +112,58 @@ __global__ void __launch_bounds__(256) k_prolong(DevGrid coarse, DevGrid fine, i
 }
 
 // Prolongation over 8^3 leaves, a warp per fine leaf: the leaf's slot, cell
-// and coarse leaf are looked up once; lane t takes voxels 16t .. 16t + 15 (two
-// k-rows, i = t / 4, j = 2t mod 8 and + 1), whose coarse voxels are the four
-// consecutive values of one coarse row, read as one float4; the rows of x
-// move as float4s.  Each active voxel takes the same fma as in k_prolong.
+// and coarse leaf are looked up once (the next leaf's slot and cell a leaf
+// ahead); lane t takes float4s t, t + 32, t + 64 and t + 96 of the leaf, so a
+// warp access is 512 consecutive bytes.  Float4 32 h + t is half t mod 2 of row
+// (2h + t / 16, t / 2 mod 8), and its coarse voxels are two consecutive values
+// of coarse row (h, t / 4 mod 4).  Each active voxel takes the same fma as in
+// k_prolong.  Bound by the load latency of a leaf's chain and by L1 wavefronts:
+// with 16 consecutive voxels a lane, whose accesses touch a line per lane, ten
+// V-cycles of the 512^3 band took 1326 us, not 1245.
 __global__ void __launch_bounds__(256) k_prolong8(DevGrid coarse, DevGrid fine, int f_src, int f_dst, float w)
 {
     chained_entry();
-    const long long n = fine.ctrl->list_n;
+    const int n = fine.ctrl->list_n;
     const int Rf = fine.R, Rc = coarse.R;
     const float *__restrict__ y = coarse.field[f_src];
     float *__restrict__ x = fine.field[f_dst];
-    const int lane = lane_id();
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long e = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < n; e += warps) {
-        const int sf = fine.list_slot[e];
-        const int b = fine.list_b[e];
-        const int bi = b / (Rf * Rf), bj = (b / Rf) % Rf, bk = b % Rf;
+    const int lane = lane_id(), half = lane & 1, cj = (lane >> 2) & 3;
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    int sn = 0, bn = 0;
+    if (e < n) {
+        sn = fine.list_slot[e];
+        bn = fine.list_b[e];
+    }
+    while (e < n) {
+        const int sf = sn, b = bn;
+        e += warps;
+        if (e < n) {
+            sn = fine.list_slot[e];
+            bn = fine.list_b[e];
+        }
+        const int bij = b / Rf, bi = bij / Rf, bj = bij - bi * Rf, bk = b - bij * Rf;
         const int sc = coarse.root[((long long)(bi >> 1) * Rc + (bj >> 1)) * Rc + (bk >> 1)];
         if (sc < 0) continue;  // the coarse voxels read 0 (warp-uniform)
-        const uint32_t bits = (fine.mask[(long long)sf * 16 + (lane >> 1)] >> ((lane & 1) * 16)) & 0xffffu;
-        if (!bits) continue;
-        const int li = lane >> 2, lj = (2 * lane) & 7;
-        const int ci = ((bi & 1) * 8 + li) >> 1, cj = ((bj & 1) * 8 + lj) >> 1, ck0 = (bk & 1) * 4;
-        const float4 yv = *reinterpret_cast<const float4 *>(y + ((long long)sc << 9) + (ci * 8 + cj) * 8 + ck0);
-        const float yk[4] = {yv.x, yv.y, yv.z, yv.w};
-        float4 *xp = reinterpret_cast<float4 *>(x + ((long long)sf << 9) + lane * 16);
+        float4 *xp = reinterpret_cast<float4 *>(x + ((long long)sf << 9)) + lane;
+        const uint32_t *mf = fine.mask + (long long)sf * 16 + (lane >> 3);
+        const float *yp = y + ((long long)sc << 9) + (((bi & 1) * 4) * 8 + (bj & 1) * 4 + cj) * 8 + (bk & 1) * 4 + 2 * half;
+        float4 v[4];
+        float2 c[4];
+        uint32_t bits[4];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            float4 v = xp[h];
-            float *c = reinterpret_cast<float *>(&v);
+            v[h] = xp[32 * h];
+            c[h] = *reinterpret_cast<const float2 *>(yp + 64 * h);
+            bits[h] = mf[4 * h] >> ((lane & 7) * 4);
+        }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int t = 4 * h + u;       // voxel 16 lane + t: k = t mod 8
-                if ((bits >> t) & 1u) c[u] = fmaf(w, yk[(t & 7) >> 1], c[u]);
-            }
-            xp[h] = v;
+        for (int h = 0; h < 4; ++h) {
+            if (bits[h] & 1u) v[h].x = fmaf(w, c[h].x, v[h].x);
+            if (bits[h] & 2u) v[h].y = fmaf(w, c[h].x, v[h].y);
+            if (bits[h] & 4u) v[h].z = fmaf(w, c[h].y, v[h].z);
+            if (bits[h] & 8u) v[h].w = fmaf(w, c[h].y, v[h].w);
+            if (bits[h] & 15u) xp[32 * h] = v[h];
         }
     }
 }

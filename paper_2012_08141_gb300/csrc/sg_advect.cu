@@ -456,17 +456,16 @@ void launch_L(const DevGrid &g, cudaStream_t s, AdvectArgs a, int ctas)
     const bool wide = (unsigned long long)(g.cap + 1) * (L * L * L) > 0x7fffffffull;
     if constexpr (MODE != 2) {
         if (a.vel4 && !wide) {
-            if (L == 8 && MODE == 0) {
+            if constexpr (L == 8 && MODE == 0) {
                 if (a.lo[0]) launch_block<0, true>(g, s, a, ctas / 8);
                 else launch_block<0, false>(g, s, a, ctas / 8);
-                return;
+            } else if constexpr (L == 8) {
+                if (a.lo[0]) launch_block<1, true>(g, s, a, ctas / 8);
+                else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
+            } else {
+                if (a.lo[0]) launch_LBO<L, MODE, true, int, true>(g, s, a, ctas);
+                else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
             }
-            if (L == 8 && MODE == 1 && a.lo[0]) {
-                launch_block<1, true>(g, s, a, ctas / 8);
-                return;
-            }
-            if (a.lo[0]) launch_LBO<L, MODE, true, int, true>(g, s, a, ctas);
-            else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
             return;
         }
     }

@@ -240,7 +240,8 @@ __device__ __forceinline__ BsPoly bs_poly(int t)
 __device__ __forceinline__ float bs_eval(const BsPoly &c, float f) { return fmaf(fmaf(c.a2, f, c.a1), f, c.a0); }
 
 // ---------------------------------------------------------------------------
-// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3), shared by the binned P2G and the fused G2P2G.  CTAs of six warps.
+// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3), shared by the
+// binned P2G and the fused G2P2G.  CTAs of six warps.
 //
 // The chunk's particles lie in shared memory as float4 records
 //   PIC   r0 = (f_i, f_j, z0, z2)  r1 = (v0, v1, v2, z1)

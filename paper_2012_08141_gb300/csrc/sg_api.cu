@@ -992,11 +992,12 @@ int do_flush(sg_grid *g)
                 if (!(rc = ensure_p2g_scratch(g, o.n))) {
                     // the same particles binned before: rebin from their last order
                     const bool rebin = g->p2g_x == o.p0 && g->p2g_n == o.n;
-                    const int k = g->dry ? p2g_launches(g->dev)
-                                         : launch_p2g_binned(g->dev, g->stream, (const float *)o.p0,
-                                                             (const float *)o.p1, (const float *)o.p3, o.n, o.f0,
-                                                             o.i0, o.i1, rebin, g->lc);
-                    g->stats.launches += k - 1;
+                    if (!g->dry &&
+                        (rc = cuda_check(launch_p2g_binned(g->dev, g->stream, (const float *)o.p0, (const float *)o.p1,
+                                                           (const float *)o.p3, o.n, o.f0, o.i0, o.i1, rebin, g->lc),
+                                         "binned p2g")))
+                        break;
+                    g->stats.launches += p2g_launches(g->dev) - 1;
                     rc = after_launch(g, "binned p2g");
                     g->p2g_x = o.p0;
                     g->p2g_n = o.n;
@@ -1013,9 +1014,11 @@ int do_flush(sg_grid *g)
                 ++i;
                 break;
             case OP_G2P2G:
-                if (!g->dry)
-                    launch_g2p2g(o.peer->dev, g->dev, o.bins->dev, g->stream, (float *)o.p1, (float *)o.p2, o.n, o.f0,
-                                 o.i0, o.f1, o.i1, o.i2, g->lc);
+                if (!g->dry &&
+                    (rc = cuda_check(launch_g2p2g(o.peer->dev, g->dev, o.bins->dev, g->stream, (float *)o.p1,
+                                                  (float *)o.p2, o.n, o.f0, o.i0, o.f1, o.i1, o.i2, g->lc),
+                                     "g2p2g")))
+                    break;
                 rc = after_launch(g, "g2p2g");
                 if (!rc) rc = bump_structure(g);
                 g->stats.act_launched++;

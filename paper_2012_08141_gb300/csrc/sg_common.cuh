@@ -1,5 +1,6 @@
 // sg_common.cuh -- small device helpers shared by the libsgrid kernels.
 #pragma once
+#include <atomic>
 #include <cstdint>
 #include "sg_device.h"
 
@@ -94,6 +95,25 @@ template <typename... P, typename... A>
 inline void launch_drained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
 {
     launch_kernel(false, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
+}
+
+// CTAs per SM of a kernel with `bytes` of dynamic shared memory, more than the
+// 48 KB that every kernel may use: it is allowed them on the current device
+// first.  Both belong to a device, so what is known is kept for each (threads
+// may race to fill an entry; they store the same).
+constexpr int kMaxDevices = 64;
+template <typename K>
+inline cudaError_t resident_per_sm(K *kernel, int threads, int bytes, std::atomic<int> (&known)[kMaxDevices], int *per)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && dev < kMaxDevices && (*per = known[dev].load(std::memory_order_relaxed)) > 0) return e;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, kernel, threads, bytes);
+    if (e == cudaSuccess && *per < 1) e = cudaErrorInvalidConfiguration;
+    if (e != cudaSuccess) cudaGetLastError();  // returned, not left for a later check
+    else if (dev < kMaxDevices) known[dev].store(*per, std::memory_order_relaxed);
+    return e;
 }
 
 // Mark the grid's structure as changed (an activation set a new bit or

@@ -277,8 +277,7 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
                          int sum_slot, const LaunchCfg &lc);
 
 // ---- particle kernels (sg_particle.cu) ----
-// Binned P2G (count, allocate, scan, order, accumulate per bin); returns the
-// number of kernels launched.  A bin is a 4^3 block of base nodes: a leaf, or
+// Binned P2G (count, allocate, scan, order, accumulate per bin).  A bin is a 4^3 block of base nodes: a leaf, or
 // an eighth of an 8^3 leaf (numbered by leaf, then by octant).  Needs
 // bin_count / bin_off (p2g_words(p2g_bins) each), bin_reach
 // (p2g_words(R^3)), tile_sum (a word per kBinTile bin words), perm and
@@ -290,9 +289,10 @@ int p2g_launches(const DevGrid &g);  // kernels of one binned P2G
 // C: NULL for PIC, else the APIC matrices (n x 9 FP32, row-major).
 // rebin: the particle order of the last binning of the same particles is
 // valid in g.perm; the new order is built from it in g.perm_alt (fewer
-// conflicting count atomics) and the two are swapped in g.
-int launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v, const float *C, long long n,
-                      float pmass, int f_mass, int f_mom0, bool rebin, const LaunchCfg &lc);
+// conflicting count atomics) and the two are swapped in g.  An error (nothing
+// launched) when the device refuses the gather's shared memory.
+cudaError_t launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v, const float *C, long long n,
+                              float pmass, int f_mass, int f_mom0, bool rebin, const LaunchCfg &lc);
 void launch_grid_update(const DevGrid &g, cudaStream_t s, int f_mass, int f_mom0, float dt,
                         float gz, int bound, const LaunchCfg &lc);
 // binned: use the bins of the last binned P2G over the same particles (the
@@ -387,8 +387,9 @@ void launch_prolong(const DevGrid &coarse, const DevGrid &fine, cudaStream_t s, 
 // ---- fused G2P2G (sg_g2p2g.cu) ----
 // APIC G2P from src (velocities f_vel0..+2) then APIC P2G with activation
 // into dst (f_mass, f_mom0..+2), C kept on chip; the particles visited in the
-// order and bins of the last binned P2G held by `bins` (src or dst).
-void launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
-                  long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc);
+// order and bins of the last binned P2G held by `bins` (src or dst).  An error
+// (nothing launched) when the device refuses its shared memory.
+cudaError_t launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
+                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc);
 
 }  // namespace sg

@@ -26,7 +26,6 @@
 // out-of-domain bin, goes node by node through the two grids; one whose new
 // base has left the bin's cells is scattered into dst by a warp, with the same
 // in-kernel allocation.
-#include <atomic>
 #include "sg_particle.cuh"
 
 namespace sg {
@@ -447,30 +446,27 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
 }
 
 template <int L>
-void launch_g2p2g_L(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
-                    float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int num_sms)
+cudaError_t launch_g2p2g_L(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x,
+                           float *v, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int num_sms)
 {
     constexpr int bytes = (int)sizeof(G2P2GSmem);
-    static std::atomic<int> resident;  // CTAs per SM; threads may race to fill it
-    int per = resident.load(std::memory_order_relaxed);
-    if (!per) {
-        cudaFuncSetAttribute(k_g2p2g<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_g2p2g<L>, kBinThreads, bytes) != cudaSuccess || per < 1)
-            per = 1;
-        resident.store(per, std::memory_order_relaxed);
-    }
+    static std::atomic<int> known[kMaxDevices];
+    int per = 0;
+    const cudaError_t e = resident_per_sm(k_g2p2g<L>, kBinThreads, bytes, known, &per);
+    if (e != cudaSuccess) return e;
     launch_chained(k_g2p2g<L>, per * num_sms, kBinThreads, bytes, s, src, dst, bins.bin_list, bins.bin_off, bins.bin_count,
                    bins.perm, &bins.ctrl->bins_used, x, v, dt, f_vel0, pmass, f_mass, f_mom0);
+    return cudaSuccess;
 }
 
 }  // namespace
 
-void launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
-                  long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc)
+cudaError_t launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
+                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc)
 {
-    if (n <= 0) return;
-    if (dst.L == 4) launch_g2p2g_L<4>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
-    else launch_g2p2g_L<8>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
+    if (n <= 0) return cudaSuccess;
+    if (dst.L == 4) return launch_g2p2g_L<4>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
+    return launch_g2p2g_L<8>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
 }
 
 }  // namespace sg

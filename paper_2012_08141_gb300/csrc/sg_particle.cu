@@ -7,7 +7,6 @@
 // C is stored row-major, 9 floats per particle: (C d)_a = sum_b C[3a+b] d_b.
 // For quadratic B-splines sum_n w d d^T = dx^2/4 I, so the APIC G2P matrix is
 // C = (4/dx^2) sum_n w v_n d^T with d = node - x_p = ((a,b,c) - fx) dx.
-#include <atomic>
 #include <utility>
 #include "sg_particle.cuh"
 
@@ -662,20 +661,23 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
     if (changed) mark_dirty(g);
 }
 
+// CTAs of the gather over these bins, or the error of a device that refuses its
+// shared memory.
 template <int L, bool APIC>
-static void launch_gather(const DevGrid &g, cudaStream_t s, const float *x, const float *v, const float *C, float pmass,
-                           int f_mass, int f_mom0, const LaunchCfg &lc)
+static cudaError_t gather_ctas(int num_sms, int *ctas)
 {
-    constexpr int bytes = (int)sizeof(GatherSmem<APIC>);
-    static std::atomic<int> resident;  // CTAs per SM; threads may race to fill it
-    int per = resident.load(std::memory_order_relaxed);
-    if (!per) {
-        cudaFuncSetAttribute(k_p2g_gather<L, APIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_p2g_gather<L, APIC>, kBinThreads, bytes) != cudaSuccess || per < 1)
-            per = 1;
-        resident.store(per, std::memory_order_relaxed);
-    }
-    launch_chained(k_p2g_gather<L, APIC>, per * lc.num_sms, kBinThreads, bytes, s, g, x, v, C, pmass, f_mass, f_mom0);
+    static std::atomic<int> known[kMaxDevices];
+    int per = 0;
+    const cudaError_t e = resident_per_sm(k_p2g_gather<L, APIC>, kBinThreads, (int)sizeof(GatherSmem<APIC>), known, &per);
+    *ctas = per * num_sms;
+    return e;
+}
+
+template <int L, bool APIC>
+static void launch_gather(const DevGrid &g, cudaStream_t s, int ctas, const float *x, const float *v, const float *C,
+                          float pmass, int f_mass, int f_mom0)
+{
+    launch_chained(k_p2g_gather<L, APIC>, ctas, kBinThreads, sizeof(GatherSmem<APIC>), s, g, x, v, C, pmass, f_mass, f_mom0);
 }
 
 // ---------------------------------------------------------------------------
@@ -723,9 +725,13 @@ int launch_sort_particles(DevGrid &g, cudaStream_t s, float *x, float *v, float 
 
 int p2g_launches(const DevGrid &g) { return p2g_words(p2g_bins(g.R, g.lg2)) / kBinTile > kMaxOwnTiles ? 7 : 6; }
 
-int launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v, const float *C, long long n,
-                      float pmass, int f_mass, int f_mom0, bool rebin, const LaunchCfg &lc)
+cudaError_t launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v, const float *C, long long n,
+                              float pmass, int f_mass, int f_mom0, bool rebin, const LaunchCfg &lc)
 {
+    int gctas = 0;
+    const cudaError_t e = g.L == 4 ? (C ? gather_ctas<4, true>(lc.num_sms, &gctas) : gather_ctas<4, false>(lc.num_sms, &gctas))
+                                   : (C ? gather_ctas<8, true>(lc.num_sms, &gctas) : gather_ctas<8, false>(lc.num_sms, &gctas));
+    if (e != cudaSuccess) return e;
     const int ntiles = (int)(p2g_words(p2g_bins(g.R, g.lg2)) / kBinTile), alloc_ctas = alloc_needed_ctas(g);
     const bool scanned = ntiles > kMaxOwnTiles;
     long long pblocks = (n + 255) / 256;
@@ -745,14 +751,14 @@ int launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const float *v
         launch_chained(k_p2g_perm, (unsigned)pblocks, 256, 0, s, g, n);
     }
     if (g.L == 4) {
-        if (C) launch_gather<4, true>(g, s, x, v, C, pmass, f_mass, f_mom0, lc);
-        else launch_gather<4, false>(g, s, x, v, C, pmass, f_mass, f_mom0, lc);
+        if (C) launch_gather<4, true>(g, s, gctas, x, v, C, pmass, f_mass, f_mom0);
+        else launch_gather<4, false>(g, s, gctas, x, v, C, pmass, f_mass, f_mom0);
     } else {
-        if (C) launch_gather<8, true>(g, s, x, v, C, pmass, f_mass, f_mom0, lc);
-        else launch_gather<8, false>(g, s, x, v, C, pmass, f_mass, f_mom0, lc);
+        if (C) launch_gather<8, true>(g, s, gctas, x, v, C, pmass, f_mass, f_mom0);
+        else launch_gather<8, false>(g, s, gctas, x, v, C, pmass, f_mass, f_mom0);
     }
     std::swap(g.perm, g.perm_alt);  // the gather's cell order
-    return p2g_launches(g);
+    return cudaSuccess;
 }
 
 }  // namespace sg

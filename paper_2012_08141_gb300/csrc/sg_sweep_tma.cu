@@ -676,12 +676,9 @@ bool tma_encode_maps(const float *field, long long cap, void *out)
 int launch_batch_tma(const BatchGrid *items, int n_grids, int total_tri, float coef, double *acc, int num_sms,
                      cudaStream_t s)
 {
-    static std::atomic<int> attr_set{0};
-    if (!attr_set.load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(k_batch_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaSmem) != cudaSuccess)
-            return 1;
-        attr_set.store(1, std::memory_order_release);
-    }
+    static std::atomic<int> known[kMaxDevices];
+    int per = 0;
+    if (resident_per_sm(k_batch_tma, kTmaWarps * 32, kTmaSmem, known, &per) != cudaSuccess) return 1;
     k_batch_tma<<<sweep_tma_ctas(num_sms), kTmaWarps * 32, kTmaSmem, s>>>(items, n_grids, total_tri, coef, acc);
     return 0;
 }
@@ -694,13 +691,11 @@ void launch_tma_tasks(const DevGrid &g, cudaStream_t s, const LaunchCfg &lc)
 
 int launch_sweep_tma(const DevGrid &g, cudaStream_t s, int src, int dst, float coef, int sum_slot, const LaunchCfg &lc)
 {
-    static std::atomic<int> attr_set{0};
-    if (!attr_set.load(std::memory_order_acquire)) {
-        if (cudaFuncSetAttribute(k_sweep_tma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(k_sweep_tma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmaSmem) != cudaSuccess)
-            return 1;
-        attr_set.store(1, std::memory_order_release);
-    }
+    static std::atomic<int> known[2][kMaxDevices];
+    int per = 0;
+    if ((sum_slot >= 0 ? resident_per_sm(k_sweep_tma<true>, kTmaWarps * 32, kTmaSmem, known[1], &per)
+                       : resident_per_sm(k_sweep_tma<false>, kTmaWarps * 32, kTmaSmem, known[0], &per)) != cudaSuccess)
+        return 1;
     TmaMaps maps;
     if (!make_maps(g.field[src], g.cap, maps)) return 2;
     if (sum_slot >= 0)

@@ -1,0 +1,90 @@
+"""CPU tests of the library's host side over a fake CUDA runtime
+(fake_cudart.cpp linked with the library's objects): what it asks of the
+runtime on several devices, while a stream is recorded and after refused calls.
+Kernels do not run; their launches are logged."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import pytest
+
+import paper_2012_08141_gb300 as sg
+from paper_2012_08141_gb300 import build as sgbuild
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    sgbuild.build(force=sgbuild.is_stale() or not all(
+        os.path.exists(os.path.join(sgbuild.BUILD, s.replace(".cu", ".o"))) for s in sgbuild.SOURCES))
+    objs = [os.path.join(sgbuild.BUILD, s.replace(".cu", ".o")) for s in sgbuild.SOURCES]
+    out = str(tmp_path_factory.mktemp("fake") / "libsgrid_fake.so")
+    include = os.path.join(os.path.dirname(os.path.dirname(sgbuild.nvcc())), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", f"-I{include}",
+                    os.path.join(HERE, "fake_cudart.cpp")] + objs + ["-o", out], check=True)
+    real = sg.load_library()
+    lib = ctypes.CDLL(out)
+    for name in sg.header_functions():
+        fn, ref = getattr(lib, name), getattr(real, name)
+        fn.argtypes, fn.restype = ref.argtypes, ref.restype
+    lib.fake_log.restype = lib.sg_last_error.restype = ctypes.c_char_p
+    return lib
+
+
+class Grid:
+    """A grid over the fake runtime: the C calls, errors as codes."""
+
+    def __init__(self, lib, device=0, stream=None, lg2=2, fields=4):
+        self.lib, self.h = lib, ctypes.c_void_p()
+        lib.fake_device(device)
+        d = sg.SgDesc(64, lg2, fields, 4, 512, 0, 0)
+        self.rc = lib.sg_create(ctypes.byref(d), stream, ctypes.byref(self.h))
+
+    def __call__(self, name, *args):
+        return getattr(self.lib, name)(self.h, *args)
+
+    def log(self, *names):
+        """How often each of the kernels was launched since the last look."""
+        text = self.lib.fake_log().decode().split(";")
+        self.lib.fake_clear_log()
+        return [sum(n in t for t in text) for n in names]
+
+
+def _particles(n):
+    return [ctypes.cast((ctypes.c_float * (k * n))(), ctypes.c_void_p) for k in (3, 3, 9)]
+
+
+@pytest.mark.parametrize("lg2", [2, 3])
+@pytest.mark.parametrize("affine", [False, True])
+def test_particle_transfers_on_every_device(lib, lg2, affine):
+    """Each device's first P2G and G2P2G allow their shared memory there."""
+    x, v, C = _particles(10)
+    for device in (0, 1, 3, 0):
+        a, b = Grid(lib, device, lg2=lg2), Grid(lib, device, lg2=lg2)
+        a.log()
+        assert a("sg_p2g_apic", x, v, C if affine else None, 10, 1.0, 0, 1) == 0
+        assert a("sg_flush") == 0, lib.sg_last_error()
+        assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == 0, lib.sg_last_error()
+        assert a.log("k_p2g_gather", "k_g2p2g") == [1, 1]
+        assert a("sg_destroy") == b("sg_destroy") == 0
+    lib.fake_device(0)
+
+
+def test_refused_shared_memory_is_an_error(lib):
+    """A device that refuses the shared memory: an error, nothing launched, and
+    the same call passes once it is allowed."""
+    x, v, _ = _particles(10)
+    g = Grid(lib, 7)
+    g.log()
+    lib.fake_refuse_attributes(1)
+    assert g("sg_p2g", x, v, 10, 1.0, 0, 1) == 0
+    assert g("sg_flush") == sg.SG_ERR_CUDA
+    lib.fake_refuse_attributes(0)
+    assert g.log("k_") == [0]
+    assert g("sg_p2g", x, v, 10, 1.0, 0, 1) == 0
+    assert g("sg_flush") == 0, lib.sg_last_error()
+    assert g.log("k_p2g_bin", "k_p2g_gather") == [1, 1]
+    assert g("sg_destroy") == 0
+    lib.fake_device(0)

@@ -989,9 +989,13 @@ int do_flush(sg_grid *g)
                 rc = run_advect_run(g, i);
                 break;
             case OP_P2G:
-                if (!(rc = ensure_p2g_scratch(g, o.n))) {
-                    // the same particles binned before: rebin from their last order
+                if (capturing(g)) rc = bump_structure(g);  // refused before anything is recorded
+                if (!rc && !(rc = ensure_p2g_scratch(g, o.n))) {
+                    // the same particles binned before: rebin from their last order,
+                    // which is no longer one until all of the new one is launched
                     const bool rebin = g->p2g_x == o.p0 && g->p2g_n == o.n;
+                    g->p2g_x = nullptr;
+                    g->p2g_n = 0;
                     if (!g->dry &&
                         (rc = cuda_check(launch_p2g_binned(g->dev, g->stream, (const float *)o.p0, (const float *)o.p1,
                                                            (const float *)o.p3, o.n, o.f0, o.i0, o.i1, rebin, g->lc),
@@ -999,10 +1003,12 @@ int do_flush(sg_grid *g)
                         break;
                     g->stats.launches += p2g_launches(g->dev) - 1;
                     rc = after_launch(g, "binned p2g");
+                }
+                if (!rc) rc = bump_structure(g);
+                if (!rc) {
                     g->p2g_x = o.p0;
                     g->p2g_n = o.n;
                 }
-                if (!rc) rc = bump_structure(g);
                 g->stats.act_launched++;
                 ++i;
                 break;
@@ -1014,7 +1020,8 @@ int do_flush(sg_grid *g)
                 ++i;
                 break;
             case OP_G2P2G:
-                if (!g->dry &&
+                if (capturing(g)) rc = bump_structure(g);  // refused before anything is recorded
+                if (!rc && !g->dry &&
                     (rc = cuda_check(launch_g2p2g(o.peer->dev, g->dev, o.bins->dev, g->stream, (float *)o.p1,
                                                   (float *)o.p2, o.n, o.f0, o.i0, o.f1, o.i1, o.i2, g->lc),
                                      "g2p2g")))

@@ -88,3 +88,51 @@ def test_refused_shared_memory_is_an_error(lib):
     assert g.log("k_p2g_bin", "k_p2g_gather") == [1, 1]
     assert g("sg_destroy") == 0
     lib.fake_device(0)
+
+
+@pytest.mark.parametrize("refused", ["recording", "device"])
+def test_refused_binning_leaves_no_order(lib, refused):
+    """A P2G that was refused (in a recording, or by the device) has put no
+    particle order in memory: nothing of it is launched or recorded, the next
+    P2G bins from the positions, G2P takes the input order, and G2P2G and the
+    reordering are refused."""
+    x, v, _ = _particles(10)
+    stream = ctypes.c_void_p(4096)
+    a, b = Grid(lib, 0, stream), Grid(lib, 0, stream)
+    a.log()
+    assert a("sg_p2g", x, v, 10, 1.0, 0, 1) == 0
+    if refused == "recording":
+        assert lib.sg_graph_begin(stream) == 0
+        assert a("sg_flush") == sg.SG_ERR_INVALID
+        graph = ctypes.c_void_p()
+        assert lib.sg_graph_end(stream, ctypes.byref(graph)) == lib.sg_graph_destroy(graph) == 0
+    else:
+        lib.fake_device(8)
+        lib.fake_refuse_attributes(1)
+        assert a("sg_flush") == sg.SG_ERR_CUDA
+        lib.fake_refuse_attributes(0)
+        lib.fake_device(0)
+    assert a.log("k_") == [0]
+    assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == sg.SG_ERR_INVALID
+    assert a("sg_sort_particles", x, v, None, None, 10) == 0 and a("sg_flush") == sg.SG_ERR_INVALID
+    assert a("sg_g2p", x, v, 10, 0.1, 1) == a("sg_flush") == 0
+    assert a.log("k_g2p_binned", "k_g2p") == [0, 1]
+    for rebin in (0, 1):
+        assert a("sg_p2g", x, v, 10, 1.0, 0, 1) == a("sg_flush") == 0, lib.sg_last_error()
+        assert a.log("k_p2g_rebin", "k_p2g_bin") == [rebin, 1 - rebin]
+    assert a("sg_destroy") == b("sg_destroy") == 0
+
+
+def test_recorded_g2p2g_records_nothing(lib):
+    x, v, _ = _particles(10)
+    stream = ctypes.c_void_p(4096)
+    a, b = Grid(lib, 0, stream), Grid(lib, 0, stream)
+    assert a("sg_p2g", x, v, 10, 1.0, 0, 1) == a("sg_flush") == 0
+    a.log()
+    assert lib.sg_graph_begin(stream) == 0
+    assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == sg.SG_ERR_INVALID
+    assert a.log("k_g2p2g") == [0]
+    graph = ctypes.c_void_p()
+    assert lib.sg_graph_end(stream, ctypes.byref(graph)) == lib.sg_graph_destroy(graph) == 0
+    assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == 0, lib.sg_last_error()
+    assert a("sg_destroy") == b("sg_destroy") == 0

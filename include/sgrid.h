@@ -399,7 +399,8 @@ int sg_write_field(sg_grid *g, int32_t f, const float *host_vals, int64_t n_leav
  * SG_ERR_INVALID, nothing written); every inactive voxel of the listed
  * leaves is set to 0.  The host buffer may be reused when the call returns.
  * read: *n_active receives the count; if it exceeds cap nothing is copied
- * and SG_ERR_INVALID is returned. */
+ * and SG_ERR_INVALID is returned.  A read that returns an error of the queued
+ * work (pool exhausted, a wait that gave up) has written nothing. */
 int sg_write_field_active(sg_grid *g, int32_t f, const float *host_vals, int64_t n_active);
 int sg_read_field_active(sg_grid *g, int32_t f, int64_t cap, int64_t *n_active, float *host_vals);
 
@@ -457,7 +458,8 @@ int sg_graph_destroy(sg_graph *graph);
  * changed). */
 int sg_write_structure(sg_grid *g, int64_t n_leaves, const int32_t *leaf_b, const uint32_t *masks);
 
-/* Implicit sync, then copy result slots [0, n) to host memory.  Passage:
+/* Implicit sync, then copy result slots [0, n) to host memory (nothing if the
+ * sync returns an error).  Passage:
  * Sec. 7.1 (a device-to-host transfer flushes the queue and synchronizes);
  * the slots hold reductions such as those of the stencil_reduction
  * microbenchmark (Supp. Sec. 1). */

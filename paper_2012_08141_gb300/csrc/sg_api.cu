@@ -110,7 +110,8 @@ struct sg_grid {
     sg_stats stats{};
     int latched = SG_OK;
     std::vector<void *> blocks;
-    Ctrl *host_ctrl = nullptr;  // pinned
+    Ctrl *host_ctrl = nullptr;  // pinned, and behind it room for host_sums reduction results
+    long long host_sums = 0;
     size_t staging_bytes = 0;
     long long perm_cap = 0;  // particles the binned-P2G order array holds
     void *sort_tmp = nullptr;  // particle reordering scratch, 36 bytes per particle
@@ -136,6 +137,11 @@ struct sg_grid {
 };
 
 namespace {
+
+// Reduction results that a sync brings with the control block (32 KB; a grid
+// with more slots reads them after the sync).
+constexpr long long kHostSums = 4096;
+constexpr size_t kHostSumsAt = (sizeof(Ctrl) + 15) / 16 * 16;
 
 void *dev_alloc(sg_grid *g, size_t bytes)
 {
@@ -1122,16 +1128,20 @@ int run_checks(sg_grid *g, sg_check_report *r, bool with_list)
     return SG_OK;
 }
 
-// Flush, wait, read the control block; latch and clear device errors.
-// The end of a sync: wait for everything launched on the grid's stream, then
-// return the first latched error.
+// Wait for everything launched on the grid's stream and bring the control block.
+int read_ctrl(sg_grid *g)
+{
+    const int rc = cuda_check(cudaMemcpyAsync(g->host_ctrl, g->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, g->stream),
+                              "read control block");
+    return rc ? rc : cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
+}
+
+// The end of a sync: wait, latch and clear device errors, and return the first
+// latched one.
 int finish_sync(sg_grid *g)
 {
     int rc;
-    if ((rc = cuda_check(cudaMemcpyAsync(g->host_ctrl, g->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, g->stream),
-                         "read control block")))
-        return rc;
-    if ((rc = cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize"))) return rc;
+    if ((rc = read_ctrl(g))) return rc;
     const int bits = g->host_ctrl->err;
     if (bits) {
         cudaMemsetAsync(&g->dev.ctrl->err, 0, sizeof(int32_t), g->stream);
@@ -1160,13 +1170,14 @@ int finish_sync(sg_grid *g)
     return out;
 }
 
+// Flush, wait, read the control block; the first latched error.
 int do_sync(sg_grid *g)
 {
     const int rc = do_flush(g);
     return rc || g->dry ? rc : finish_sync(g);
 }
 
-// Implicit sync with a current list (reads need list order).
+// Flush and make the list current (reads need list order), without a wait.
 int flush_with_list(sg_grid *g)
 {
     if (g->dry) return fail(SG_ERR_INVALID, "a dry-run grid holds no data");
@@ -1180,6 +1191,7 @@ int flush_with_list(sg_grid *g)
     return SG_OK;
 }
 
+// Implicit sync with a current list.
 int sync_with_list(sg_grid *g)
 {
     const int rc = flush_with_list(g);
@@ -1198,9 +1210,8 @@ int ensure_staging(sg_grid *g)
     return SG_OK;
 }
 
-// Packed positions of every list entry's active voxels (a current list of n
-// entries); returns their total through *total (implicit wait).  Kept while
-// the structure is unchanged: the list version keys them.
+// Launch the packed positions of every list entry's active voxels (a current
+// list of n entries); their total goes to ctrl->act_total.
 int queue_active_offsets(sg_grid *g, long long n)
 {
     if (!g->act_off) {
@@ -1217,6 +1228,8 @@ int queue_active_offsets(sg_grid *g, long long n)
 // device dirty flag, read at the last sync, is clear).
 bool offsets_kept(const sg_grid *g) { return g->act_ver == g->list_ver && g->act_ver != 0 && g->host_ctrl->dirty == 0; }
 
+// The packed positions, kept while the structure is unchanged (the list version
+// keys them); returns their total through *total (implicit wait).
 int active_offsets(sg_grid *g, long long n, long long *total)
 {
     if (offsets_kept(g)) {
@@ -1254,11 +1267,7 @@ int run_write_staged(sg_grid *g, const Op &o)
         // the list length, on the host: wait for the work launched so far and
         // read the control block (no flush -- this runs inside one; device
         // errors stay latched for the next sync)
-        if ((rc = cuda_check(cudaMemcpyAsync(g->host_ctrl, g->dev.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost,
-                                             g->stream),
-                             "read control block")) ||
-            (rc = cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize")))
-            return rc;
+        if ((rc = read_ctrl(g))) return rc;
     }
     const long long n = g->host_ctrl->list_n;
     if (n > 0 && (rc = active_offsets(g, n, &total))) return rc;
@@ -1357,7 +1366,8 @@ int grid_create(const sg_desc *desc, void *cuda_stream, sg_grid **out, bool init
             return fail(SG_ERR_OOM, "field allocation");
         }
     }
-    if (cudaMallocHost((void **)&g->host_ctrl, sizeof(Ctrl)) != cudaSuccess) {
+    g->host_sums = std::min<long long>(desc->max_sums, kHostSums);
+    if (cudaMallocHost((void **)&g->host_ctrl, kHostSumsAt + sizeof(double) * g->host_sums) != cudaSuccess) {
         cudaGetLastError();
         dev_free_all(g);
         delete g;
@@ -1964,57 +1974,49 @@ int sg_write_field_active(sg_grid *g, int32_t f, const float *host_vals, int64_t
 // (from a sync since it was generated): the gather is launched behind the
 // flushed work, and a single wait covers both and brings the control block, so
 // a batch's results of 64 grids cost 64 waits, not 128, each with the GPU busy
-// up to it (20 batched steps and the 64 reads 5764 -> 5520 us).
+// up to it (20 batched steps and the 64 reads 5764 -> 5520 us).  The gather
+// compares the count with the buffer's capacity and looks at the error word on
+// the device, so a call that fails has written nothing.
 int sg_read_field_active(sg_grid *g, int32_t f, int64_t cap, int64_t *n_active, float *host_vals)
 {
     if (!g || !valid_field(g, f) || cap < 0 || !n_active) return fail(SG_ERR_INVALID, "bad arguments");
     int rc = flush_with_list(g);
     if (rc) return rc;
-    bool waited = false;  // everything launched so far is done and had no error
+    bool waited = false;  // everything flushed is done and had no error
     if (g->ctrl_ver != g->list_ver || (g->desc.flags & SG_CREATE_CHECK)) {
         if ((rc = finish_sync(g))) return rc;
         waited = true;
     }
     const long long n = g->host_ctrl->list_n;
-    float *direct = nullptr;
-    if (n > 0 && !offsets_kept(g)) {
-        // the count comes back with the values when they go in place: the
-        // gather compares it with the buffer's capacity on the device
-        direct = (float *)mapped_host(host_vals, sizeof(float) * size_t(cap));
-        if (direct) {
-            if ((rc = queue_active_offsets(g, n))) return rc;
-            launch_gather_active(g->dev, g->stream, g->phys[f], direct, n, cap, g->act_off, g->act_tsum, g->lc);
-            if ((rc = after_launch(g, "gather active")) || (rc = finish_sync(g))) return rc;
-            g->act_ver = g->list_ver;
-            g->act_total = g->host_ctrl->act_total;
-            *n_active = g->act_total;
-            if (g->act_total > cap)
-                return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels", (long long)cap,
-                            g->act_total);
-            return SG_OK;
-        }
+    const bool kept = n > 0 && offsets_kept(g), compute = n > 0 && !kept;
+    if (compute && (rc = queue_active_offsets(g, n))) return rc;
+    // in place: as far as the host knows, the call may write all of the leaves
+    const long long most = std::min<long long>(cap, kept ? g->act_total : n * g->dev.L * g->dev.L * g->dev.L);
+    float *direct = n > 0 ? (float *)mapped_host(host_vals, sizeof(float) * size_t(most)) : nullptr;
+    if (direct) {
+        launch_gather_active(g->dev, g->stream, g->phys[f], direct, n, cap, g->act_off, g->act_tsum, g->lc);
+        if ((rc = after_launch(g, "gather active"))) return rc;
     }
-    long long total = 0;
-    if (n > 0 && (rc = active_offsets(g, n, &total))) return rc;
+    if (!waited || compute || direct)
+        if ((rc = waited ? read_ctrl(g) : finish_sync(g))) return rc;
+    if (compute) {
+        g->act_ver = g->list_ver;
+        g->act_total = g->host_ctrl->act_total;
+    }
+    const long long total = n > 0 ? g->act_total : 0;
     *n_active = total;
-    if (total > cap || total == 0 || !host_vals) {
-        if (!waited && (rc = finish_sync(g))) return rc;
-        if (total > cap)
-            return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels", (long long)cap,
-                        total);
-        return total == 0 ? SG_OK : fail(SG_ERR_INVALID, "null buffer");
-    }
-    const size_t bytes = sizeof(float) * size_t(total);
-    direct = (float *)mapped_host(host_vals, bytes);
-    if (!direct && (rc = ensure_staging(g))) return rc;
-    launch_gather_active(g->dev, g->stream, g->phys[f], direct ? direct : g->dev.staging, n, cap, g->act_off,
-                         g->act_tsum, g->lc);
-    if ((rc = after_launch(g, "gather active"))) return rc;
-    if (!direct && (rc = cuda_check(cudaMemcpyAsync(host_vals, g->dev.staging, bytes, cudaMemcpyDeviceToHost,
-                                                    g->stream),
-                                    "copy active values")))
+    if (total > cap)
+        return fail(SG_ERR_INVALID, "buffer holds %lld values, the grid has %lld active voxels", (long long)cap, total);
+    if (direct || total == 0) return SG_OK;
+    if (!host_vals) return fail(SG_ERR_INVALID, "null buffer");
+    if ((rc = ensure_staging(g))) return rc;
+    launch_gather_active(g->dev, g->stream, g->phys[f], g->dev.staging, n, cap, g->act_off, g->act_tsum, g->lc);
+    if ((rc = after_launch(g, "gather active")) ||
+        (rc = cuda_check(cudaMemcpyAsync(host_vals, g->dev.staging, sizeof(float) * size_t(total), cudaMemcpyDeviceToHost,
+                                         g->stream),
+                         "copy active values")))
         return rc;
-    return finish_sync(g);
+    return cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
 }
 
 struct sg_graph {
@@ -2119,10 +2121,21 @@ int sg_read_sums(sg_grid *g, double *host, int64_t n)
     if (g->dry) return fail(SG_ERR_INVALID, "a dry-run grid holds no data");
     int rc = do_flush(g);
     if (rc) return rc;
-    if (n > 0 &&
-        (rc = cuda_check(cudaMemcpyAsync(host, g->dev.sums, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream), "copy sums")))
+    // one wait for the flushed work and the results, which go to the caller
+    // once the sync has found no error; more than fit are copied after it
+    double *sums = (double *)((char *)g->host_ctrl + kHostSumsAt);
+    const bool along = n > 0 && n <= g->host_sums;
+    if (along &&
+        (rc = cuda_check(cudaMemcpyAsync(sums, g->dev.sums, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream), "copy sums")))
         return rc;
-    return finish_sync(g);
+    if ((rc = finish_sync(g)) || n == 0) return rc;
+    if (along) {
+        std::memcpy(host, sums, sizeof(double) * n);
+        return SG_OK;
+    }
+    if ((rc = cuda_check(cudaMemcpyAsync(host, g->dev.sums, sizeof(double) * n, cudaMemcpyDeviceToHost, g->stream), "copy sums")))
+        return rc;
+    return cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
 }
 
 int sg_set_stencil_variant(sg_grid *g, int32_t variant)

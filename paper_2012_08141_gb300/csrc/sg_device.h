@@ -171,7 +171,8 @@ void launch_scatter_field(const DevGrid &g, cudaStream_t s, int f, const float *
 // launch_active_offsets leaves the packed position of each list entry's first
 // active voxel in off[e] + tsum[e / kOffTile] and the total in
 // tsum[ceil(n / kOffTile)] and ctrl->act_total.  src holds exactly that many
-// values; the gather writes nothing if they are more than out's cap.
+// values; the gather writes nothing if they are more than out's cap or the error
+// word is set.
 constexpr int kOffTile = 1024;
 void launch_active_offsets(const DevGrid &g, cudaStream_t s, long long n, long long *off, long long *tsum);
 void launch_scatter_active(const DevGrid &g, cudaStream_t s, int f, const float *src, long long total,

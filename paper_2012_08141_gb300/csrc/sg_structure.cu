@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(256) k_gather_active(DevGrid g, int f, float *
 {
     chained_entry();
     const long long total = tsum[ntiles];
-    if (total > cap) return;
+    if (total > cap || g.ctrl->err) return;
     constexpr int V = L * L * L, W = V / 32, CAP = 4096, T = CAP / V;
     __shared__ float s_val[CAP];
     const long long n = g.ctrl->list_n;

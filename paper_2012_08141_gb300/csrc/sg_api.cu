@@ -1390,8 +1390,7 @@ int grid_create(const sg_desc *desc, void *cuda_stream, sg_grid **out, bool init
     Ctrl c{};
     c.dirty = 1;
     std::memcpy(g->host_ctrl, &c, sizeof c);
-    launch_init_grid(s, sp, d.ctrl, c, g->lc);
-    rc = cuda_check(cudaPeekAtLastError(), "grid initialisation");
+    rc = cuda_check(launch_init_grid(s, sp, d.ctrl, c, g->lc), "grid initialisation");
     if (!rc && init_sync) rc = cuda_check(cudaStreamSynchronize(s), "init sync");
     if (rc) {
         cudaStreamSynchronize(s);  // the queued initialisation still writes the blocks

@@ -62,7 +62,7 @@ __device__ __forceinline__ void chained_entry()
 }
 
 template <typename... P, typename... A>
-inline void launch_kernel(bool chained, void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s,
+inline cudaError_t launch_kernel(bool chained, void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s,
                           A &&...args)
 {
     cudaLaunchConfig_t cfg{};
@@ -75,13 +75,13 @@ inline void launch_kernel(bool chained, void (*kernel)(P...), long long ctas, in
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = chained ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 template <typename... P, typename... A>
-inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+inline cudaError_t launch_chained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
 {
-    launch_kernel(true, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
+    return launch_kernel(true, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
 }
 
 // For a resident kernel whose CTAs together want more shared memory than the
@@ -92,9 +92,9 @@ inline void launch_chained(void (*kernel)(P...), long long ctas, int threads, si
 // when the kernels before it have drained; the next one may still be chained
 // to it.
 template <typename... P, typename... A>
-inline void launch_drained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
+inline cudaError_t launch_drained(void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s, A &&...args)
 {
-    launch_kernel(false, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
+    return launch_kernel(false, kernel, ctas, threads, smem, s, static_cast<A &&>(args)...);
 }
 
 // CTAs per SM of a kernel with `bytes` of dynamic shared memory, more than the

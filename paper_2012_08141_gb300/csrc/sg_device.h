@@ -264,7 +264,7 @@ struct InitSpans {
     } span[6 + kMaxFields];
     int n;
 };
-void launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc);
+cudaError_t launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc);
 
 // ---- device-side fill with the counter-based generator (sg_structure.cu) ----
 void launch_fill_hash(const DevGrid &g, cudaStream_t s, int f, unsigned long long seed, const LaunchCfg &lc);

@@ -676,12 +676,12 @@ __global__ void __launch_bounds__(256) k_init_grid(const __grid_constant__ InitS
     }
 }
 
-void launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc)
+cudaError_t launch_init_grid(cudaStream_t s, const InitSpans &spans, Ctrl *ctrl, const Ctrl &state, const LaunchCfg &lc)
 {
     long long bytes = 0;
     for (int q = 0; q < spans.n; ++q) bytes += spans.span[q].bytes;
     const long long ctas = (bytes + 4095) / 4096, most = lc.num_sms * 8LL;
-    launch_chained(k_init_grid, ctas < most ? ctas : most, 256, 0, s, spans, ctrl, state);
+    return launch_chained(k_init_grid, ctas < most ? ctas : most, 256, 0, s, spans, ctrl, state);
 }
 
 // A group of G = min(32, L^3 / 4) threads fills one leaf, four k-adjacent

@@ -136,3 +136,16 @@ def test_recorded_g2p2g_records_nothing(lib):
     assert lib.sg_graph_end(stream, ctypes.byref(graph)) == lib.sg_graph_destroy(graph) == 0
     assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == 0, lib.sg_last_error()
     assert a("sg_destroy") == b("sg_destroy") == 0
+
+
+def test_create_beside_an_earlier_error(lib):
+    """An error that an earlier call left with the thread (here a read from a
+    stream being recorded) is not the new grid's."""
+    a = Grid(lib, 0, ctypes.c_void_p(4096))
+    assert lib.sg_graph_begin(ctypes.c_void_p(4096)) == 0
+    assert a("sg_read_sums", (ctypes.c_double * 4)(), 4) == sg.SG_ERR_CUDA
+    b = Grid(lib, 0, ctypes.c_void_p(8192))
+    assert b.rc == 0, lib.sg_last_error()
+    graph = ctypes.c_void_p()
+    assert lib.sg_graph_end(ctypes.c_void_p(4096), ctypes.byref(graph)) == lib.sg_graph_destroy(graph) == 0
+    assert a("sg_destroy") == b("sg_destroy") == 0

@@ -42,7 +42,18 @@ struct AdvectArgs {
     float *lo[kMaxAdvectChannels];
     float *hi[kMaxAdvectChannels];
     const float4 *vel4;               // packed velocity, or null (read the three fields)
+    const uint32_t *vmax;             // with k_advect_block: the largest packed component (see below)
 };
+
+// Does every voxel move by less than a cell over h?  k_advect_block runs if so
+// and k_advect if not; both are launched and the other returns at once (vmax:
+// bits of a non-negative float, a NaN above all).  Longer steps leave the staged
+// block, and a voxel that does is traced twice: with the block kernel alone
+// three channels on the 256^3 tube took 352 us a step up to a cell, 485 at 1.6
+// cells and 692 at 5 (k_advect: 405, 405 and 410; with the choice 355, 403 and
+// 405).  The results are the same either way, so a largest component left over
+// from an earlier packing costs time only.
+__device__ __forceinline__ bool steps_within_a_cell(const AdvectArgs &A) { return __uint_as_float(__ldg(A.vmax)) * fabsf(A.h) < 1.f; }
 
 // Slot of the leaf holding cell (ci, cj, ck), relative to the list entry's
 // leaf (bi, bj, bk): through the neighbour table within one leaf, else the root.
@@ -252,6 +263,7 @@ template <int L, int C, int MODE, bool BND, typename Off, bool PK>
 __global__ void __launch_bounds__(256, 4) k_advect(DevGrid g, AdvectArgs A)
 {
     chained_entry();
+    if (L == 8 && PK && A.vmax && steps_within_a_cell(A)) return;
     constexpr int V = L * L * L, LG2 = (L == 8) ? 3 : 2;
     const long long n = g.ctrl->list_n;
     __shared__ int s_nb[8][27];
@@ -349,6 +361,7 @@ __global__ void __launch_bounds__(256, 5) k_advect_block(const __grid_constant__
     __shared__ float4 s_v[kBlkCells];
     __shared__ float s_q[C][kBlkCells];
     __shared__ int s_nb[27];
+    if (!steps_within_a_cell(A)) return;
     const int n = g.ctrl->list_n, R = g.R, tid = threadIdx.x;
     const float h = MODE == 0 ? A.h : -A.h;
     int nb = tid < 27 && (int)blockIdx.x < n ? g.nbr[blockIdx.x * 27LL + tid] : 0;  // an entry ahead
@@ -431,20 +444,21 @@ __global__ void __launch_bounds__(256, 5) k_advect_block(const __grid_constant__
     }
 }
 
-template <int MODE, bool BND>
-void launch_block(const DevGrid &g, cudaStream_t s, const AdvectArgs &a, int num_sms)
-{
-    if (a.C == 1) launch_drained(k_advect_block<1, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
-    else if (a.C == 2) launch_drained(k_advect_block<2, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
-    else launch_drained(k_advect_block<3, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
-}
-
 template <int L, int MODE, bool BND, typename Off, bool PK>
 void launch_LBO(const DevGrid &g, cudaStream_t s, const AdvectArgs &a, int ctas)
 {
     if (a.C == 1) launch_chained(k_advect<L, 1, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
     else if (a.C == 2) launch_chained(k_advect<L, 2, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
     else launch_chained(k_advect<L, 3, MODE, BND, Off, PK>, ctas, 256, 0, s, g, a);
+}
+
+template <int MODE, bool BND>
+void launch_block(const DevGrid &g, cudaStream_t s, const AdvectArgs &a, int num_sms)
+{
+    if (a.C == 1) launch_drained(k_advect_block<1, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
+    else if (a.C == 2) launch_drained(k_advect_block<2, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
+    else launch_drained(k_advect_block<3, MODE, BND>, num_sms * 5, 256, 0, s, g, a);
+    launch_LBO<8, MODE, BND, int, true>(g, s, a, num_sms * 8);
 }
 
 template <int L, int MODE>
@@ -456,20 +470,25 @@ void launch_L(const DevGrid &g, cudaStream_t s, AdvectArgs a, int ctas)
     const bool wide = (unsigned long long)(g.cap + 1) * (L * L * L) > 0x7fffffffull;
     if constexpr (MODE != 2) {
         if (a.vel4 && !wide) {
-            if constexpr (L == 8 && MODE == 0) {
-                if (a.lo[0]) launch_block<0, true>(g, s, a, ctas / 8);
-                else launch_block<0, false>(g, s, a, ctas / 8);
-            } else if constexpr (L == 8) {
-                if (a.lo[0]) launch_block<1, true>(g, s, a, ctas / 8);
-                else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
-            } else {
-                if (a.lo[0]) launch_LBO<L, MODE, true, int, true>(g, s, a, ctas);
-                else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
+            if constexpr (L == 8) {
+                if (a.vmax && (MODE == 0 || a.lo[0])) {
+                    if constexpr (MODE == 0) {
+                        if (a.lo[0]) launch_block<0, true>(g, s, a, ctas / 8);
+                        else launch_block<0, false>(g, s, a, ctas / 8);
+                    } else {
+                        launch_block<1, true>(g, s, a, ctas / 8);
+                    }
+                    return;
+                }
             }
+            a.vmax = nullptr;
+            if (a.lo[0]) launch_LBO<L, MODE, true, int, true>(g, s, a, ctas);
+            else launch_LBO<L, MODE, false, int, true>(g, s, a, ctas);
             return;
         }
     }
     a.vel4 = nullptr;
+    a.vmax = nullptr;
     if (a.lo[0]) {
         if (wide) launch_LBO<L, MODE, true, long long, false>(g, s, a, ctas);
         else launch_LBO<L, MODE, true, int, false>(g, s, a, ctas);
@@ -480,33 +499,51 @@ void launch_L(const DevGrid &g, cudaStream_t s, AdvectArgs a, int ctas)
 }
 
 // Packed velocity: vel4[slot * L^3 + l] = (u, v, w, 0) of fields v0..v0+2 for
-// every listed leaf (the zero leaf's block is zero from its allocation).
+// every listed leaf (the zero leaf's block is zero from its allocation), and
+// the largest component in *vmax, zero before; *next is zeroed for the packing
+// after this one.
 template <int L>
-__global__ void __launch_bounds__(256) k_pack_velocity(DevGrid g, int v0, float4 *__restrict__ vel4)
+__global__ void __launch_bounds__(256, 8) k_pack_velocity(const __grid_constant__ DevGrid g, int v0, float4 *__restrict__ vel4, uint32_t *vmax,
+                                                          uint32_t *next)
 {
     chained_entry();
+    __shared__ uint32_t s_max[8];
+    uint32_t most = 0;
     constexpr int V = L * L * L, LG2 = (L == 8) ? 3 : 2;
     const long long n = g.ctrl->list_n;
     const float *__restrict__ u = g.field[v0], *__restrict__ v = g.field[v0 + 1], *__restrict__ w = g.field[v0 + 2];
+#pragma unroll 1  // unrolled it needs more than the 32 registers of eight CTAs per SM
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < n * V;
          q += (long long)gridDim.x * blockDim.x) {
         const long long idx = ((long long)g.list_slot[q >> (3 * LG2)] << (3 * LG2)) + (q & (V - 1));
-        vel4[idx] = make_float4(__ldg(u + idx), __ldg(v + idx), __ldg(w + idx), 0.f);
+        const float4 a = make_float4(__ldg(u + idx), __ldg(v + idx), __ldg(w + idx), 0.f);
+        vel4[idx] = a;
+        most = max(max(most, __float_as_uint(fabsf(a.x))), max(__float_as_uint(fabsf(a.y)), __float_as_uint(fabsf(a.z))));
+    }
+    most = __reduce_max_sync(kFull, most);
+    if (lane_id() == 0) s_max[threadIdx.x >> 5] = most;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) most = max(most, s_max[q]);
+        if (most > *(volatile uint32_t *)vmax) atomicMax(vmax, most);
+        if (blockIdx.x == 0) *next = 0;
     }
 }
 
 }  // namespace
 
-void launch_pack_velocity(const DevGrid &g, cudaStream_t s, int v0, float4 *vel4, const LaunchCfg &lc)
+void launch_pack_velocity(const DevGrid &g, cudaStream_t s, int v0, float4 *vel4, uint32_t *vmax, uint32_t *next,
+                          const LaunchCfg &lc)
 {
     const int ctas = lc.num_sms * 8;
-    if (g.L == 8) launch_chained(k_pack_velocity<8>, ctas, 256, 0, s, g, v0, vel4);
-    else launch_chained(k_pack_velocity<4>, ctas, 256, 0, s, g, v0, vel4);
+    if (g.L == 8) launch_chained(k_pack_velocity<8>, ctas, 256, 0, s, g, v0, vel4, vmax, next);
+    else launch_chained(k_pack_velocity<4>, ctas, 256, 0, s, g, v0, vel4, vmax, next);
 }
 
 void launch_advect_group(const DevGrid &g, cudaStream_t s, int mode, int C, const int *dst, const int *src,
                          const int *qhat, const int *qtil, int v0, float h, float *const *lo, float *const *hi,
-                         const float4 *vel4, const LaunchCfg &lc)
+                         const float4 *vel4, const uint32_t *vmax, const LaunchCfg &lc)
 {
     AdvectArgs a{};
     a.C = C;
@@ -521,6 +558,7 @@ void launch_advect_group(const DevGrid &g, cudaStream_t s, int mode, int C, cons
     a.v0 = v0;
     a.h = h;
     a.vel4 = vel4;
+    a.vmax = vmax;
     const int ctas = lc.num_sms * 8;
     if (g.L == 8) {
         if (mode == 0) launch_L<8, 0>(g, s, a, ctas);

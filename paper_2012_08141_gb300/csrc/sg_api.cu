@@ -78,6 +78,11 @@ struct Op {
 // leaves, after this many sweeps without its run records.
 constexpr long long kSingleRunsLeaves = 8192;
 constexpr int kSingleRunsAfter = 2;
+// A fused advection over 8^3 leaves stages leaves in shared memory from this many
+// on (the count at the last sync; unknown: it does).  It gains 4 us a step per
+// thousand leaves and costs 4 us a step, the launches of the kernels that are
+// not chosen (960 leaves, three channels: 38.4 us a step without, 40.7 with).
+constexpr long long kAdvectBlockLeaves = 1024;
 
 struct sg_grid {
     sg_desc desc{};
@@ -125,6 +130,7 @@ struct sg_grid {
     long long act_total = 0;
     float *adv_lo[3] = {}, *adv_hi[3] = {}; // advection clamp bounds, (cap + 1) * L^3 each (allocated at first use)
     float4 *adv_vel4 = nullptr;             // packed advection velocity, (cap + 1) * L^3 (allocated at first use)
+    unsigned adv_packs = 0;                 // which of the two words behind it holds its largest component
     // staged uploads (sg_stage_active): two slots filled on a copy stream of
     // the grid's own, each consumed by a queued scatter
     cudaStream_t copy_stream = nullptr;
@@ -698,11 +704,15 @@ int run_advect_run(sg_grid *g, size_t &i)
     auto ensure_vel4 = [&]() -> bool {
         if (g->dry || g->adv_vel4) return true;
         const size_t per_leaf = size_t(g->dev.L) * g->dev.L * g->dev.L;
-        g->adv_vel4 = (float4 *)dev_alloc(g, sizeof(float4) * size_t(g->dev.cap + 1) * per_leaf);
+        g->adv_vel4 = (float4 *)dev_alloc(g, sizeof(float4) * size_t(g->dev.cap + 1) * per_leaf + 2 * sizeof(uint32_t));
         if (!g->adv_vel4) return false;
-        // the zero leaf's block: never written by the packing, read as zeros
-        return cudaMemsetAsync(g->adv_vel4 + size_t(g->dev.cap) * per_leaf, 0, sizeof(float4) * per_leaf,
+        // the zero leaf's block: never written by the packing, read as zeros;
+        // behind it the largest component of every other packing
+        return cudaMemsetAsync(g->adv_vel4 + size_t(g->dev.cap) * per_leaf, 0, sizeof(float4) * per_leaf + 2 * sizeof(uint32_t),
                                g->stream) == cudaSuccess;
+    };
+    auto packed_max = [&](unsigned k) {
+        return (uint32_t *)(g->adv_vel4 + size_t(g->dev.cap + 1) * g->dev.L * g->dev.L * g->dev.L) + k;
     };
     auto launch = [&](int mode, const std::vector<int> &ops, const std::vector<int> &macs) -> int {
         int r2;
@@ -714,7 +724,10 @@ int run_advect_run(sg_grid *g, size_t &i)
                 if (!ensure_vel4()) {
                     pack_v0 = -1;  // without the memory: read the three fields
                 } else {
-                    if (!g->dry) launch_pack_velocity(g->dev, g->stream, pack_v0, g->adv_vel4, g->lc);
+                    g->adv_packs ^= 1;
+                    if (!g->dry)
+                        launch_pack_velocity(g->dev, g->stream, pack_v0, g->adv_vel4, packed_max(g->adv_packs),
+                                             packed_max(g->adv_packs ^ 1), g->lc);
                     g->stats.velocity_packs++;
                     packed = true;
                     if ((r2 = after_launch(g, "velocity packing"))) return r2;
@@ -790,9 +803,10 @@ int run_advect_run(sg_grid *g, size_t &i)
                 for (int c = 0; c < 3; ++c) lo[c] = hi[c] = nullptr;
         }
         if (bnd) g->stats.bounds_reused += (mode == 0) ? 0 : C;
+        const bool small = g->known_leaves > 0 && g->known_leaves < kAdvectBlockLeaves;
         if (!g->dry)
             launch_advect_group(g->dev, g->stream, mode, C, dst, src, qh, qt, f.i0, h, bnd ? lo : nullptr,
-                                bnd ? hi : nullptr, vel4, g->lc);
+                                bnd ? hi : nullptr, vel4, vel4 && !small ? packed_max(g->adv_packs) : nullptr, g->lc);
         g->stats.ops_fused += (int64_t)(mode == 1 ? 2 * C : C) - 1;
         for (int c : ops) done[c] = 1;
         for (int c : macs) done[c] = 1;

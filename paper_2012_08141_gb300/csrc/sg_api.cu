@@ -633,11 +633,12 @@ static bool intersects(const std::vector<int> &a, const std::vector<int> &b)
 // The run queue[i .. end) of advection ops as fused launches (Sec. 6.4,
 // Supp. Sec. 2).  The ops' dependencies come from their read / write sets
 // (the state-flow edges between them); ops whose dependencies are all issued
-// are ready and mutually independent.  Ready backward advections whose output
-// q~ a correction reads at the voxel (an element-wise connection) are fused
-// with that correction, q~ then stored only if a later op reads it (Sec. 6.5);
-// other ready ops with the same velocity and step are grouped, up to three
-// channels per launch.  Without fusion each op is a launch, in queue order.
+// are ready and mutually independent.  A ready backward advection of a
+// correction's q^ whose output q~ it reads at the voxel (an element-wise
+// connection) is fused with that correction, q~ then stored only if a later op
+// reads it (Sec. 6.5); other ready ops with the same velocity and step are
+// grouped, up to three channels per launch.  Without fusion each op is a launch,
+// in queue order.
 int run_advect_run(sg_grid *g, size_t &i)
 {
     int rc;
@@ -830,7 +831,8 @@ int run_advect_run(sg_grid *g, size_t &i)
             if (done[a] || o.kind != OP_ADVECT || o.f0 >= 0.f || !issued(a, -1)) continue;
             for (int m = a + 1; m < n; ++m) {
                 const Op &c = g->queue[i + m];
-                if (done[m] || c.kind != OP_MAC || c.i2 != o.dst || c.i0 != o.i0 || c.f0 != -o.f0 || !issued(m, a))
+                if (done[m] || c.kind != OP_MAC || c.i2 != o.dst || c.i1 != o.src || c.i0 != o.i0 || c.f0 != -o.f0 ||
+                    !issued(m, a))
                     continue;
                 if (!ops.empty()) {
                     const Op &o0 = g->queue[i + ops[0]];

@@ -106,9 +106,9 @@ typedef struct sg_desc {
 } sg_desc;
 
 typedef struct sg_stats {
-    int64_t launches;        /* device kernels launched (copies not counted; the two
-                                of which the device picks one as a fused advection
-                                over 8^3 leaves count as one) */
+    int64_t launches;        /* device kernels launched (copies not counted; where the
+                                device picks one of two, as for a fused advection over
+                                8^3 leaves and a G2P2G, they count as one) */
     int64_t listgen_run;     /* list-generation kernels launched */
     int64_t listgen_removed; /* list generations removed on the host (Sec. 6.2) */
     int64_t act_launched;    /* activation kernels launched */

@@ -123,6 +123,7 @@ struct sg_grid {
     long long sort_cap = 0;
     const void *p2g_x = nullptr;  // positions and count the order array was built for
     long long p2g_n = 0;
+    mutable int g2p2g_turn = 0;  // fused G2P2G launches over that order, modulo 3
     unsigned long long *chk_cnt = nullptr;  // invariant-check counters (allocated at the first check)
     long long *act_off = nullptr;           // active-voxel transfer offsets, [cap] and [cap / kOffTile + 2]
     long long *act_tsum = nullptr;
@@ -1028,6 +1029,7 @@ int do_flush(sg_grid *g)
                 }
                 if (!rc) rc = bump_structure(g);
                 if (!rc) {
+                    g->g2p2g_turn = 0;
                     g->p2g_x = o.p0;
                     g->p2g_n = o.n;
                 }
@@ -1045,9 +1047,11 @@ int do_flush(sg_grid *g)
                 if (capturing(g)) rc = bump_structure(g);  // refused before anything is recorded
                 if (!rc && !g->dry &&
                     (rc = cuda_check(launch_g2p2g(o.peer->dev, g->dev, o.bins->dev, g->stream, (float *)o.p1,
-                                                  (float *)o.p2, o.n, o.f0, o.i0, o.f1, o.i1, o.i2, g->lc),
+                                                  (float *)o.p2, o.n, o.f0, o.i0, o.f1, o.i1, o.i2,
+                                                  o.bins->g2p2g_turn, g->lc),
                                      "g2p2g")))
                     break;
+                o.bins->g2p2g_turn = (o.bins->g2p2g_turn + 1) % 3;
                 rc = after_launch(g, "g2p2g");
                 if (!rc) rc = bump_structure(g);
                 g->stats.act_launched++;

@@ -51,7 +51,8 @@ struct Ctrl {
     int32_t bins_used;    // leaves holding particles in the last binned P2G
     long long act_total;  // active voxels of the last active-offset scan
     uint32_t rr_ticket;   // run-record tiles handed out (zeroed before each region-mask launch)
-    int32_t pad[1];
+    int32_t moved[3];     // fused G2P2G over the last binning: particles found outside their bin's cells,
+                          // by launch in turn
 };
 
 struct DevGrid {
@@ -391,8 +392,10 @@ void launch_prolong(const DevGrid &coarse, const DevGrid &fine, cudaStream_t s, 
 // APIC G2P from src (velocities f_vel0..+2) then APIC P2G with activation
 // into dst (f_mass, f_mom0..+2), C kept on chip; the particles visited in the
 // order and bins of the last binned P2G held by `bins` (src or dst).  An error
-// (nothing launched) when the device refuses its shared memory.
+// (nothing launched) when the device refuses its shared memory.  turn: how many
+// such launches there were since the binning, modulo 3.
 cudaError_t launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
-                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc);
+                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int turn,
+                         const LaunchCfg &lc);
 
 }  // namespace sg

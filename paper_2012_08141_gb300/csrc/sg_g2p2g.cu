@@ -18,14 +18,16 @@
 //   2. per particle: G2P from the staged block, store x', v'; count it in its
 //      new base cell and store its P2G record of the new position;
 //   3. counting sort by new base cell;
-//   4. sums by columns of cells, as in the binned P2G (bin_columns);
-//   5. flush the touched nodes o .. o+5: the dst leaves they fall in are
-//      allocated in-kernel if null (see ensure_leaf), bits set, 4 FP32 atomics
-//      per node.
+//   4. sums by columns of cells, as in the binned P2G (bin_columns), over the
+//      bin's own cells or, once many particles have moved there, those around;
+//   5. flush the touched nodes o .. o+5 (o-1 .. o+6): the dst leaves they fall
+//      in are allocated in-kernel if null (see ensure_leaf), bits set, 4 FP32
+//      atomics per node.
 // A particle whose old base has left [o-1, o+4], and every particle of the
 // out-of-domain bin, goes node by node through the two grids; one whose new
-// base has left the bin's cells is scattered into dst by a warp, with the same
-// in-kernel allocation.
+// base is further out than those cells is scattered into dst by a warp, with
+// the same in-kernel allocation.
+#include <type_traits>
 #include "sg_particle.cuh"
 
 namespace sg {
@@ -173,6 +175,226 @@ __device__ __forceinline__ bool scatter_particle(const DevGrid &g, Spline sx, Sp
 }
 
 // ---------------------------------------------------------------------------
+// Sorting and summing of a chunk's new positions, in two forms.  Particles move
+// on from step to step and one binning serves many, so at first nearly all are
+// in their bin's own 4^3 cells and later many are not.
+//   k_g2p2g<L, false>  BinSort and bin_columns, as the binned P2G: a particle
+//                      outside the own cells is added to dst by a warp.
+//   k_g2p2g<L, true>   MovedSort: cells 0 .. 63 are the bin's own, 64 .. 215 the
+//                      152 around them (base o - 1 .. o + 4), 216 holds what has
+//                      gone further.  Up to kFewMoved particles in the cells
+//                      around, they are added to dst by a warp each, like those
+//                      of 216; with more, the chunk is summed by 36 columns of
+//                      six cells, the bin's own 16 and then the 20 around them,
+//                      onto the 8^3 nodes o - 1 .. o + 6.
+// Each launch counts the particles that it finds outside the own cells; from the
+// next launch over the same binning on, the second form runs if they were more
+// than one in kMovedShare.  Both are launched and the other returns at once.  2M
+// particles, 10 a cell, that have moved by 0 / 0.03 / 0.1 / 0.25 / 1 cell since
+// the binning: the first form takes 232 / 272 / 344 / 459 / 941 us, the second
+// (more shared memory, less L1) 257 / 302 / 342 / 349 / 347.
+// ---------------------------------------------------------------------------
+constexpr int kMovedShare = 16;
+constexpr int kOwnCells = 64, kFarCell = 216, kFewMoved = 24;
+constexpr int kMovedBuf = 36 * 9 * 8;  // float4 [column][lane][node]
+
+struct MovedSort {
+    int cnt[kFarCell + 1];    // particles per cell; zero between chunks
+    int start[224];           // their places in idx
+    uint32_t prev[36], all[36];  // nodes that the particles of each column (6 x 6, of six cells) reach, before / after this chunk
+    int slot[8 + 27];         // blocks o / 4 + {0, 1}^3 and, for moved particles, o / 4 + {-1, 0, 1}^3
+    uint32_t bits[2 * (8 + 27)]; // touched nodes of those blocks, i, j, k in order
+    int moved;                // this chunk is summed by the 36 columns
+    int outer;                // a chunk of this bin was
+};
+
+// Cell (i, j, k), each 0 .. 5 from o - 1.
+__device__ __forceinline__ int moved_cell(int i, int j, int k)
+{
+    if ((unsigned)(i - 1) < 4u && (unsigned)(j - 1) < 4u) {
+        if ((unsigned)(k - 1) < 4u) return ((i - 1) * 4 + j - 1) * 4 + k - 1;
+        return kOwnCells + (k == 0 ? 120 : 136) + (i - 1) * 4 + j - 1;
+    }
+    return kOwnCells + ((unsigned)(i - 1) < 4u ? (j == 0 ? 72 : 96) + (i - 1) * 6 + k : (i == 0 ? 0 : 36) + j * 6 + k);
+}
+
+// Exclusive scan of the cell counts (one warp), which it zeroes.
+__device__ __forceinline__ void moved_scan(MovedSort &s)
+{
+    constexpr int PER = 7;  // 32 x 7 >= 217; an odd stride has no bank conflicts
+    const int lane = lane_id();
+    int c[PER], tot = 0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        const int cell = PER * lane + q;
+        c[q] = cell <= kFarCell ? s.cnt[cell] : 0;
+        tot += c[q];
+        if (cell <= kFarCell) s.cnt[cell] = 0;
+    }
+    int run = warp_incl_scan(tot) - tot;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+        s.start[PER * lane + q] = run;  // start[217 ..]: the end
+        run += c[q];
+    }
+    __syncwarp();
+    const bool moved = s.start[kFarCell] - s.start[kOwnCells] > kFewMoved;
+    if (lane == 0) {
+        s.moved = moved;
+        if (moved) s.outer = 1;
+    }
+    for (int col = lane; col < 36; col += 32) {
+        const int i = col / 6, j = col - 6 * i;
+        const bool own = (unsigned)(i - 1) < 4u && (unsigned)(j - 1) < 4u;
+        uint32_t now = 0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (moved || (own && (unsigned)(k - 1) < 4u)) {
+                const int cell = moved_cell(i, j, k);
+                if (s.start[cell + 1] > s.start[cell]) now |= 7u << k;
+            }
+        const uint32_t before = s.all[col];
+        s.prev[col] = before;
+        s.all[col] = before | now;
+    }
+}
+
+// Column sums as in bin_columns, of a chunk whose particles stayed in the bin's
+// own cells (but for the few that go by a warp each).
+template <int CAP>
+__device__ __forceinline__ void own_columns(const float4 (*rec)[CAP], const uint16_t *idx, const MovedSort &s, float4 *s_buf)
+{
+    const int lane = lane_id(), grp = lane / 9, sub = lane - 9 * grp;
+    const int own = (threadIdx.x >> 5) * 3 + grp;
+    if (grp > 2 || own > 15) return;
+    int pp = s.start[4 * own];
+    const int last = s.start[4 * own + 4];
+    if (pp >= last || last > CAP) return;
+    const int a = sub / 3, b = sub - 3 * a, col = ((own >> 2) + 1) * 6 + (own & 3) + 1;
+    const BsPoly pa = bs_poly(a), pb = bs_poly(b);
+    const uint32_t add = s.prev[col];  // nodes with sums of an earlier chunk
+    float4 *out = s_buf + (col * 9 + sub) * 8 + 1;
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
+    auto store = [&](int k, float4 n) {
+        if (add >> (k + 1) & 1u) {
+            const float4 o = out[k];
+            n = make_float4(o.x + n.x, o.y + n.y, o.z + n.z, o.w + n.w);
+        }
+        out[k] = n;
+    };
+    int next = idx[pp];
+#pragma unroll 1
+    for (int ck = 0; ck < 4; ++ck) {
+        const int end = s.start[4 * own + ck + 1];
+        while (pp < end) {
+            const int q = next;
+            next = idx[++pp];
+            column_add<true, CAP>(rec, q, pa, pb, (float)a, (float)b, n0, n1, n2);
+        }
+        store(ck, n0);
+        n0 = n1;
+        n1 = n2;
+        n2 = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    store(4, n0);
+    store(5, n1);
+}
+
+// The same over the 36 columns.
+template <int CAP>
+__device__ __noinline__ void moved_columns(const float4 (*rec)[CAP], const uint16_t *idx, const MovedSort &s, float4 *s_buf)
+{
+    const int lane = lane_id(), grp = lane / 9, sub = lane - 9 * grp;
+    if (grp > 2 || s.start[kFarCell + 1] > CAP) return;
+    const int a = sub / 3, b = sub - 3 * a;
+    const BsPoly pa = bs_poly(a), pb = bs_poly(b);
+#pragma unroll 1
+    for (int c = (threadIdx.x >> 5) * 3 + grp; c < 36; c += 18) {
+        // the bin's own 16 first, then the rows and the columns around them
+        const int col = c < 16 ? ((c >> 2) + 1) * 6 + (c & 3) + 1
+                        : c < 22 ? c - 16 : c < 28 ? c + 8 : c < 32 ? (c - 27) * 6 : (c - 31) * 6 + 5;
+        const int i = col / 6, j = col - 6 * i;
+        const uint32_t add = s.prev[col];
+        float4 *out = s_buf + (col * 9 + sub) * 8;
+        float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0;
+        auto store = [&](int k, float4 n) {
+            if (add >> k & 1u) {
+                const float4 o = out[k];
+                n = make_float4(o.x + n.x, o.y + n.y, o.z + n.z, o.w + n.w);
+            }
+            out[k] = n;
+        };
+        if (!s.all[col]) continue;
+#pragma unroll 1
+        for (int k = 0; k < 6; ++k) {
+            const int cell = moved_cell(i, j, k), end = s.start[cell + 1];
+            for (int pp = s.start[cell]; pp < end; ++pp)
+                column_add<true, CAP>(rec, idx[pp], pa, pb, (float)a, (float)b, n0, n1, n2);
+            store(k, n0);
+            n0 = n1;
+            n1 = n2;
+            n2 = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        store(6, n0);
+        store(7, n1);
+    }
+}
+
+// Does any summed particle's stencil hold node (i, j, k) (0 .. 7 from o - 1)?
+__device__ __forceinline__ bool moved_hit(const MovedSort &s, int i, int j, int k)
+{
+    uint32_t m = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            if ((unsigned)(i - a) < 6u && (unsigned)(j - b) < 6u) m |= s.all[(i - a) * 6 + (j - b)];
+    return (m >> k & 1u) != 0u;
+}
+
+// Its sums over the columns that reach it.
+__device__ __forceinline__ float4 moved_total(const MovedSort &s, const float4 *s_buf, int i, int j, int k)
+{
+    float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int ci = i - a, cj = j - b, col = ci * 6 + cj;
+            if ((unsigned)ci >= 6u || (unsigned)cj >= 6u || !(s.all[col] >> k & 1u)) continue;
+            const float4 v = s_buf[(col * 9 + a * 3 + b) * 8 + k];
+            t.x += v.x;
+            t.y += v.y;
+            t.z += v.z;
+            t.w += v.w;
+        }
+    return t;
+}
+
+// One record by a warp (cell: pack_cell's word): lane (a, b, c) < 27 forms the
+// contribution of its node base + (a, b, c); false for lanes without a node in
+// the domain.  t: weight and weighted velocity.
+template <int CAP>
+__device__ __forceinline__ bool single_node(const float4 (*rec)[CAP], int q, int cell, int oi, int oj, int ok, int N, int &i,
+                                            int &j, int &k, float4 &t)
+{
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, c = lane % 3;
+    if (lane >= 27) return false;
+    i = oi + (cell >> 20) - 512 + a;
+    j = oj + ((cell >> 10) & 1023) - 512 + b;
+    k = ok + (cell & 1023) - 512 + c;
+    if ((unsigned)i >= (unsigned)N || (unsigned)j >= (unsigned)N || (unsigned)k >= (unsigned)N) return false;
+    const float4 r0 = rec[0][q], r1 = rec[1][q], r2 = rec[2][q], r3 = rec[3][q];
+    const float w = bs_eval(bs_poly(a), r0.x) * bs_eval(bs_poly(b), r0.y) *
+                    (c == 0 ? r0.z : c == 1 ? (1.f - r0.z) - r0.w : r0.w);
+    const float ta = (float)a, tb = (float)b, tc = (float)c;
+    t = make_float4(w, w * fmaf(r1.w, ta, fmaf(r2.x, tb, fmaf(r2.y, tc, r1.x))),
+                    w * fmaf(r2.z, ta, fmaf(r2.w, tb, fmaf(r3.x, tc, r1.y))),
+                    w * fmaf(r3.y, ta, fmaf(r3.z, tb, fmaf(r3.w, tc, r1.z))));
+    return true;
+}
+
+// ---------------------------------------------------------------------------
 // The next chunk's positions come into shared memory while a chunk is worked
 // on.  A bin of several chunks deals its particles to them in turn, so each
 // chunk has its share of every column whatever the order.  A whole bin of the
@@ -182,16 +404,18 @@ __device__ __forceinline__ bool scatter_particle(const DevGrid &g, Spline sx, Sp
 // and a warp per cell: 308 us; this one at three CTAs and 96 registers,
 // spilling: 264 us).
 // ---------------------------------------------------------------------------
+template <bool AROUND>
 struct G2P2GSmem {
     static constexpr int PPT = 4, CAP = 736;
     float4 rec[4][CAP];
-    float4 buf[kBinBuf];
+    float4 buf[AROUND ? kMovedBuf : kBinBuf];
     float4 u[512];                  // src velocities of nodes o - 1 .. o + 6
     float x[3 * CAP];               // the next chunk's positions, in order
     float words[kBinWarps][96];
     int uslot[27];                  // src blocks o / 4 + {-1, 0, 1}^3
     uint16_t idx[CAP + 2];
-    BinSort sort;
+    int cell[AROUND ? CAP : 1];     // pack_cell of the records outside the bin's own cells
+    std::conditional_t<AROUND, MovedSort, BinSort> sort;
 };
 
 // One particle node by node: its G2P from src, its state, its P2G into dst.
@@ -216,16 +440,21 @@ __device__ __noinline__ bool far_particle(const DevGrid &src, const DevGrid &dst
 }
 constexpr int kFar = -2;
 
-template <int L>
+template <int L, bool AROUND>
 __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant__ DevGrid src,
                                                           const __grid_constant__ DevGrid dst,
                                                           const int32_t *bin_list, const int32_t *bin_off,
                                                           const int32_t *bin_end, const int32_t *perm,
-                                                          const int32_t *bins_used, float *x, float *v, float dt,
-                                                          int f_vel0, float pmass, int f_mass, int f_mom0)
+                                                          Ctrl *bin_ctrl, int turn, long long n, float *x, float *v,
+                                                          float dt, int f_vel0, float pmass, int f_mass, int f_mom0)
 {
     chained_entry();
-    using S = G2P2GSmem;
+    // of the three counts one is the last launch's, one this one's and one the
+    // next one's, zero then
+    if ((bin_ctrl->moved[turn] > n / kMovedShare) != AROUND) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) bin_ctrl->moved[(turn + 2) % 3] = 0;
+    int moved_here = 0;
+    using S = G2P2GSmem<AROUND>;
     constexpr int PPT = S::PPT, CAP = S::CAP;
     extern __shared__ __align__(16) unsigned char smem[];
     S &s = *reinterpret_cast<S *>(smem);
@@ -236,7 +465,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
     float *words = s.words[warp];
     const float *u0p = src.field[f_vel0], *u1p = src.field[f_vel0 + 1], *u2p = src.field[f_vel0 + 2];
     bool changed = false;
-    const int used = *bins_used;
+    const int used = bin_ctrl->bins_used;
     // particles whose stencil missed the domain when they were binned
     {
         const int oob_bin = (int)p2g_bins(R, L == 8 ? 3 : 2);
@@ -288,8 +517,15 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
         order(beg, end, 0, nch, p);
         request(p);
         if (bl + (int)gridDim.x < used) bin_of(bl + gridDim.x, nb, nbeg, nend);
-        if (threadIdx.x < 65) s.sort.cnt[threadIdx.x] = 0;
-        if (threadIdx.x < 16) s.sort.all[threadIdx.x] = s.sort.bits[threadIdx.x] = 0;
+        constexpr int OUT = AROUND ? kFarCell : kOwnCells;  // the cell of the particles that no column sums
+        auto fresh_bin = [&] {
+            if (threadIdx.x < (AROUND ? 36 : 16)) s.sort.all[threadIdx.x] = 0;
+            if (threadIdx.x < (AROUND ? 2 * (8 + 27) : 16)) s.sort.bits[threadIdx.x] = 0;
+            if constexpr (AROUND)
+                if (threadIdx.x == 0) s.sort.outer = 0;
+        };
+        for (int q = threadIdx.x; q <= OUT; q += kBinThreads) s.sort.cnt[q] = 0;
+        fresh_bin();
         if (threadIdx.x < 27) s.uslot[threadIdx.x] = slot;
         __syncthreads();
         for (;;) {
@@ -343,10 +579,13 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                         const Spline nx = bspline(xn[0], N), ny = bspline(xn[1], N), nz = bspline(xn[2], N);
                         const int ci = nx.base - oi, cj = ny.base - oj, ck = nz.base - ok;
                         if ((unsigned)(ci + 500) <= 1000u && (unsigned)(cj + 500) <= 1000u && (unsigned)(ck + 500) <= 1000u) {
-                            const bool in = (unsigned)ci < 4u && (unsigned)cj < 4u && (unsigned)ck < 4u;
-                            const int cell = in ? (ci * 4 + cj) * 4 + ck : 64;
-                            pl = cell | atomicAdd(&s.sort.cnt[cell], 1) << 7;
-                            bin_record<true, CAP>(s.rec, q, nx.fx, ny.fx, nz.fx, uu.x, uu.y, uu.z, C, dx, !in,
+                            constexpr int E = AROUND ? 1 : 0;  // cells around
+                            const bool near = (unsigned)(ci + E) < 4u + 2 * E && (unsigned)(cj + E) < 4u + 2 * E &&
+                                              (unsigned)(ck + E) < 4u + 2 * E;
+                            const int cell = near ? moved_cell(ci + 1, cj + 1, ck + 1) : OUT;
+                            pl = cell | atomicAdd(&s.sort.cnt[cell], 1) << 8;
+                            if (AROUND && cell >= kOwnCells) s.cell[AROUND ? q : 0] = __float_as_int(pack_cell(ci, cj, ck));
+                            bin_record<true, CAP>(s.rec, q, nx.fx, ny.fx, nz.fx, uu.x, uu.y, uu.z, C, dx, !AROUND && !near,
                                                   pack_cell(ci, cj, ck));
                         }
                     }
@@ -360,19 +599,34 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                     if (u == w) place[w] = pl;
             }
             __syncthreads();
-            if (warp == 0) bin_scan(s.sort);
+            if (warp == 0) {
+                if constexpr (AROUND) moved_scan(s.sort);
+                else bin_scan(s.sort);
+            }
             __syncthreads();
+            if (threadIdx.x == 0) moved_here += s.sort.start[OUT + 1] - s.sort.start[kOwnCells];
 #pragma unroll
             for (int u = 0; u < PPT; ++u)
                 if (place[u] >= 0)
-                    s.idx[s.sort.start[place[u] & 127] + (place[u] >> 7)] = (uint16_t)((u * kBinWarps + warp) * 32 + lane);
+                    s.idx[s.sort.start[place[u] & 255] + (place[u] >> 8)] = (uint16_t)((u * kBinWarps + warp) * 32 + lane);
             __syncthreads();
             if (more) request(pn);
-            bin_columns<true, CAP>(s.rec, s.idx, s.sort, s.buf);
-            for (int pp = s.sort.start[64] + warp; pp < s.sort.start[65] && pp < CAP; pp += kBinWarps) {
+            bool moved = false;
+            if constexpr (AROUND) {
+                moved = s.sort.moved != 0;
+                if (moved) moved_columns<CAP>(s.rec, s.idx, s.sort, s.buf);
+                else own_columns<CAP>(s.rec, s.idx, s.sort, s.buf);
+            } else {
+                bin_columns<true, CAP>(s.rec, s.idx, s.sort, s.buf);
+            }
+            for (int pp = s.sort.start[moved ? OUT : kOwnCells] + warp; pp < s.sort.start[OUT + 1] && pp < CAP; pp += kBinWarps) {
                 int i, j, k;
                 float4 t;
-                if (edge_node<true, CAP>(s.rec, s.idx[pp], oi, oj, ok, N, i, j, k, t))
+                const int q = s.idx[pp];
+                bool in;
+                if constexpr (AROUND) in = single_node<CAP>(s.rec, q, s.cell[q], oi, oj, ok, N, i, j, k, t);
+                else in = edge_node<true, CAP>(s.rec, q, oi, oj, ok, N, i, j, k, t);
+                if (in)
                     changed |= scatter_node(dst, i, j, k, pmass * t.x, pmass * t.y, pmass * t.z, pmass * t.w, f_mass, f_mom0);
             }
 #pragma unroll
@@ -390,25 +644,59 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                     if (nd >= kBinNodes) continue;
                     int i, j, k, blk, l;
                     bin_node(nd, i, j, k, blk, l);
-                    if (oi + i >= N || oj + j >= N || ok + k >= N || !node_hit(s.sort, i, j, k)) continue;
-                    t[h] = node_total(s.sort, s.buf, i, j, k);
+                    if (oi + i >= N || oj + j >= N || ok + k >= N) continue;
+                    if constexpr (AROUND) {
+                        if (!moved_hit(s.sort, i + 1, j + 1, k + 1)) continue;
+                        t[h] = moved_total(s.sort, s.buf, i + 1, j + 1, k + 1);
+                    } else {
+                        if (!node_hit(s.sort, i, j, k)) continue;
+                        t[h] = node_total(s.sort, s.buf, i, j, k);
+                    }
                     where[h] = blk << 6 | l;
                     atomicOr(&s.sort.bits[2 * blk + (l >> 5)], 1u << (l & 31));
                 }
+                auto add = [&](int ds, int l, float4 v) {
+                    const long long idx = block_voxel<L>(ds, l >> 4, l >> 2 & 3, l & 3);
+                    atomicAdd(dst.field[f_mass] + idx, pmass * v.x);
+                    atomicAdd(dst.field[f_mom0] + idx, pmass * v.y);
+                    atomicAdd(dst.field[f_mom0 + 1] + idx, pmass * v.z);
+                    atomicAdd(dst.field[f_mom0 + 2] + idx, pmass * v.w);
+                };
+                // the nodes o - 1 and o + 6 of a bin with particles in the cells around
+                [[maybe_unused]] auto outer_nodes = [&](auto &&take) {
+                    for (int nd = threadIdx.x; nd < 512; nd += kBinThreads) {
+                        const int i = nd >> 6, j = nd >> 3 & 7, k = nd & 7;
+                        if ((unsigned)(i - 1) < 6u && (unsigned)(j - 1) < 6u && (unsigned)(k - 1) < 6u) continue;
+                        if ((unsigned)(oi + i - 1) >= (unsigned)N || (unsigned)(oj + j - 1) >= (unsigned)N ||
+                            (unsigned)(ok + k - 1) >= (unsigned)N)
+                            continue;
+                        take(i, j, k, 8 + ((i + 3) >> 2) * 9 + ((j + 3) >> 2) * 3 + ((k + 3) >> 2),
+                             ((i + 3) & 3) << 4 | ((j + 3) & 3) << 2 | ((k + 3) & 3));
+                    }
+                };
+                bool outer = false;
+                if constexpr (AROUND) {
+                    outer = s.sort.outer != 0;
+                    if (outer)
+                        outer_nodes([&](int i, int j, int k, int blk, int l) {
+                            if (moved_hit(s.sort, i, j, k)) atomicOr(&s.sort.bits[2 * blk + (l >> 5)], 1u << (l & 31));
+                        });
+                }
                 __syncthreads();
                 if (warp == 0) {
-                    if (lane < 8) {
-                        const int ci = bi + (lane >> 2), cj = bj + ((lane >> 1) & 1), ck = bk + (lane & 1);
+                    auto leaf = [&](int blk, int ci, int cj, int ck) {
                         int ds = -1;
-                        if (s.sort.bits[2 * lane] | s.sort.bits[2 * lane + 1]) {
+                        if (s.sort.bits[2 * blk] | s.sort.bits[2 * blk + 1]) {
                             bool fresh = false;
                             ds = block_of_leaf<L>(ensure_leaf(dst, block_leaf<L>(R, ci, cj, ck), fresh), ci, cj, ck);
                             changed |= fresh;
                         }
-                        s.sort.slot[lane] = ds;
-                    }
+                        s.sort.slot[blk] = ds;
+                    };
+                    if (lane < 8) leaf(lane, bi + (lane >> 2), bj + ((lane >> 1) & 1), bk + (lane & 1));
+                    if (outer && lane < 27) leaf(8 + lane, bi + lane / 9 - 1, bj + (lane / 3) % 3 - 1, bk + lane % 3 - 1);
                     __syncwarp();
-                    changed |= set_touched<L>(dst, s.sort);
+                    changed |= set_touched<L>(dst, s.sort.slot, s.sort.bits, outer ? 35 : 8);
                     if (lane < 27) s.uslot[lane] = slot;
                 }
                 __syncthreads();
@@ -416,16 +704,16 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                 for (int h = 0; h < 2; ++h) {
                     if (where[h] < 0) continue;
                     const int ds = s.sort.slot[where[h] >> 6];
-                    if (ds < 0) continue;  // pool exhausted; the error is latched
-                    const int l = where[h] & 63;
-                    const long long idx = block_voxel<L>(ds, l >> 4, l >> 2 & 3, l & 3);
-                    atomicAdd(dst.field[f_mass] + idx, pmass * t[h].x);
-                    atomicAdd(dst.field[f_mom0] + idx, pmass * t[h].y);
-                    atomicAdd(dst.field[f_mom0 + 1] + idx, pmass * t[h].z);
-                    atomicAdd(dst.field[f_mom0 + 2] + idx, pmass * t[h].w);
+                    if (ds >= 0) add(ds, where[h] & 63, t[h]);  // else the pool is exhausted; the error is latched
                 }
+                if constexpr (AROUND)
+                    if (outer)
+                        outer_nodes([&](int i, int j, int k, int blk, int l) {
+                            const int ds = s.sort.slot[blk];
+                            if (ds >= 0 && moved_hit(s.sort, i, j, k)) add(ds, l, moved_total(s.sort, s.buf, i, j, k));
+                        });
                 __syncthreads();
-                if (threadIdx.x < 16) s.sort.all[threadIdx.x] = s.sort.bits[threadIdx.x] = 0;
+                fresh_bin();
                 if (!more) break;
                 bl += gridDim.x;
                 b = nb;
@@ -442,31 +730,37 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
             for (int u = 0; u < PPT; ++u) p[u] = pn[u];
         }
     }
+    if (moved_here) atomicAdd(&bin_ctrl->moved[(turn + 1) % 3], moved_here);
     if (changed) mark_dirty(dst);
 }
 
 template <int L>
 cudaError_t launch_g2p2g_L(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x,
-                           float *v, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int num_sms)
+                           float *v, long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int turn,
+                           int num_sms)
 {
-    constexpr int bytes = (int)sizeof(G2P2GSmem);
-    static std::atomic<int> known[kMaxDevices];
-    int per = 0;
-    const cudaError_t e = resident_per_sm(k_g2p2g<L>, kBinThreads, bytes, known, &per);
+    constexpr int bytes[2] = {(int)sizeof(G2P2GSmem<false>), (int)sizeof(G2P2GSmem<true>)};
+    static std::atomic<int> known[2][kMaxDevices];
+    int per[2];
+    cudaError_t e = resident_per_sm(k_g2p2g<L, false>, kBinThreads, bytes[0], known[0], &per[0]);
+    if (e == cudaSuccess) e = resident_per_sm(k_g2p2g<L, true>, kBinThreads, bytes[1], known[1], &per[1]);
     if (e != cudaSuccess) return e;
-    launch_chained(k_g2p2g<L>, per * num_sms, kBinThreads, bytes, s, src, dst, bins.bin_list, bins.bin_off, bins.bin_count,
-                   bins.perm, &bins.ctrl->bins_used, x, v, dt, f_vel0, pmass, f_mass, f_mom0);
+    launch_chained(k_g2p2g<L, false>, per[0] * num_sms, kBinThreads, bytes[0], s, src, dst, bins.bin_list, bins.bin_off,
+                   bins.bin_count, bins.perm, bins.ctrl, turn, n, x, v, dt, f_vel0, pmass, f_mass, f_mom0);
+    launch_chained(k_g2p2g<L, true>, per[1] * num_sms, kBinThreads, bytes[1], s, src, dst, bins.bin_list, bins.bin_off,
+                   bins.bin_count, bins.perm, bins.ctrl, turn, n, x, v, dt, f_vel0, pmass, f_mass, f_mom0);
     return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t launch_g2p2g(const DevGrid &src, const DevGrid &dst, const DevGrid &bins, cudaStream_t s, float *x, float *v,
-                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, const LaunchCfg &lc)
+                         long long n, float dt, int f_vel0, float pmass, int f_mass, int f_mom0, int turn,
+                         const LaunchCfg &lc)
 {
     if (n <= 0) return cudaSuccess;
-    if (dst.L == 4) return launch_g2p2g_L<4>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
-    return launch_g2p2g_L<8>(src, dst, bins, s, x, v, dt, f_vel0, pmass, f_mass, f_mom0, lc.num_sms);
+    if (dst.L == 4) return launch_g2p2g_L<4>(src, dst, bins, s, x, v, n, dt, f_vel0, pmass, f_mass, f_mom0, turn, lc.num_sms);
+    return launch_g2p2g_L<8>(src, dst, bins, s, x, v, n, dt, f_vel0, pmass, f_mass, f_mom0, turn, lc.num_sms);
 }
 
 }  // namespace sg

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(256) k_bin_clear(DevGrid g)
     const long long q = blockIdx.x * 256LL + threadIdx.x;
     reinterpret_cast<int4 *>(g.bin_count)[q] = make_int4(0, 0, 0, 0);
     if (q < p2g_words(p2g_bins(g.R, 2)) / 4) reinterpret_cast<int4 *>(g.bin_reach)[q] = make_int4(0, 0, 0, 0);
-    if (q == 0) g.ctrl->bins_used = 0;
+    if (q == 0) g.ctrl->bins_used = g.ctrl->moved[0] = g.ctrl->moved[1] = g.ctrl->moved[2] = 0;
 }
 
 // Particles of one bin with the reach classes `classes` (a bit each).  The
@@ -638,7 +638,7 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
             }
             __syncthreads();
             if (warp == 0) {
-                changed |= set_touched<L>(g, s.sort);
+                changed |= set_touched<L>(g, s.sort.slot, s.sort.bits, 8);
                 __syncwarp();  // the bin's shared state for the next bin
                 if (lane < 16) s.sort.all[lane] = s.sort.bits[lane] = 0;
                 if (lane < 8) s.sort.slot[lane] = slot;

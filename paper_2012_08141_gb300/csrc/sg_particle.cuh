@@ -240,8 +240,9 @@ __device__ __forceinline__ BsPoly bs_poly(int t)
 __device__ __forceinline__ float bs_eval(const BsPoly &c, float f) { return fmaf(fmaf(c.a2, f, c.a1), f, c.a0); }
 
 // ---------------------------------------------------------------------------
-// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3), shared by the
-// binned P2G and the fused G2P2G.  CTAs of six warps.
+// P2G sums of one bin of 4^3 cells (the base cells o .. o + 3), as the binned
+// P2G takes them; the fused G2P2G, whose particles have moved since they were
+// binned, has its own sort and walk around the same sums.  CTAs of six warps.
 //
 // The chunk's particles lie in shared memory as float4 records
 //   PIC   r0 = (f_i, f_j, z0, z2)  r1 = (v0, v1, v2, z1)
@@ -307,6 +308,40 @@ __device__ __forceinline__ void bin_scan(BinSort &s)
     }
 }
 
+// Record q's contribution to the three nodes of its cell in column lane (a, b)
+// (pa, pb: its weights; ta, tb: a and b).
+template <bool APIC, int CAP>
+__device__ __forceinline__ void column_add(const float4 (*rec)[CAP], int q, const BsPoly &pa, const BsPoly &pb, float ta,
+                                           float tb, float4 &n0, float4 &n1, float4 &n2)
+{
+    const float4 r0 = rec[0][q], r1 = rec[1][q];
+    const float w = bs_eval(pa, r0.x) * bs_eval(pb, r0.y);
+    const float w0 = w * r0.z, w1 = w * (APIC ? (1.f - r0.z) - r0.w : r1.w), w2 = w * r0.w;
+    float u0 = r1.x, u1 = r1.y, u2 = r1.z;
+    float m2 = 0.f, m5 = 0.f, m8 = 0.f;
+    if (APIC) {
+        const float4 r2 = rec[APIC ? 2 : 0][q], r3 = rec[APIC ? 3 : 0][q];
+        u0 = fmaf(r1.w, ta, fmaf(r2.x, tb, u0));
+        u1 = fmaf(r2.z, ta, fmaf(r2.w, tb, u1));
+        u2 = fmaf(r3.y, ta, fmaf(r3.z, tb, u2));
+        m2 = r2.y;
+        m5 = r3.x;
+        m8 = r3.w;
+    }
+    n0.x += w0;
+    n0.y = fmaf(w0, u0, n0.y);
+    n0.z = fmaf(w0, u1, n0.z);
+    n0.w = fmaf(w0, u2, n0.w);
+    n1.x += w1;
+    n1.y = fmaf(w1, APIC ? u0 + m2 : u0, n1.y);
+    n1.z = fmaf(w1, APIC ? u1 + m5 : u1, n1.z);
+    n1.w = fmaf(w1, APIC ? u2 + m8 : u2, n1.w);
+    n2.x += w2;
+    n2.y = fmaf(w2, APIC ? fmaf(2.f, m2, u0) : u0, n2.y);
+    n2.z = fmaf(w2, APIC ? fmaf(2.f, m5, u1) : u1, n2.z);
+    n2.w = fmaf(w2, APIC ? fmaf(2.f, m8, u2) : u2, n2.w);
+}
+
 // idx has CAP + 1 entries at least: a particle's place is read one ahead.
 template <bool APIC, int CAP>
 __device__ __forceinline__ void bin_columns(const float4 (*rec)[CAP], const uint16_t *idx, const BinSort &s,
@@ -338,32 +373,7 @@ __device__ __forceinline__ void bin_columns(const float4 (*rec)[CAP], const uint
         while (pp < end) {
             const int q = next;
             next = idx[++pp];
-            const float4 r0 = rec[0][q], r1 = rec[1][q];
-            const float w = bs_eval(pa, r0.x) * bs_eval(pb, r0.y);
-            const float w0 = w * r0.z, w1 = w * (APIC ? (1.f - r0.z) - r0.w : r1.w), w2 = w * r0.w;
-            float u0 = r1.x, u1 = r1.y, u2 = r1.z;
-            float m2 = 0.f, m5 = 0.f, m8 = 0.f;
-            if (APIC) {
-                const float4 r2 = rec[APIC ? 2 : 0][q], r3 = rec[APIC ? 3 : 0][q];
-                u0 = fmaf(r1.w, ta, fmaf(r2.x, tb, u0));
-                u1 = fmaf(r2.z, ta, fmaf(r2.w, tb, u1));
-                u2 = fmaf(r3.y, ta, fmaf(r3.z, tb, u2));
-                m2 = r2.y;
-                m5 = r3.x;
-                m8 = r3.w;
-            }
-            n0.x += w0;
-            n0.y = fmaf(w0, u0, n0.y);
-            n0.z = fmaf(w0, u1, n0.z);
-            n0.w = fmaf(w0, u2, n0.w);
-            n1.x += w1;
-            n1.y = fmaf(w1, APIC ? u0 + m2 : u0, n1.y);
-            n1.z = fmaf(w1, APIC ? u1 + m5 : u1, n1.z);
-            n1.w = fmaf(w1, APIC ? u2 + m8 : u2, n1.w);
-            n2.x += w2;
-            n2.y = fmaf(w2, APIC ? fmaf(2.f, m2, u0) : u0, n2.y);
-            n2.z = fmaf(w2, APIC ? fmaf(2.f, m5, u1) : u1, n2.z);
-            n2.w = fmaf(w2, APIC ? fmaf(2.f, m8, u2) : u2, n2.w);
+            column_add<APIC, CAP>(rec, q, pa, pb, ta, tb, n0, n1, n2);
         }
         store(ck, n0);
         n0 = n1;
@@ -416,30 +426,32 @@ __device__ __forceinline__ void bin_node(int nd, int &i, int &j, int &k, int &bl
     l = ((i & 3) << 4) | ((j & 3) << 2) | (k & 3);
 }
 
-// Set the touched nodes' bits in their leaves' masks (one warp; a lane per mask
-// word: two of a 4^3 leaf, four of a block in an 8^3 one).  Returns whether
-// this lane set a new one.
+// Set the touched nodes' bits of n blocks in their leaves' masks (one warp; a
+// lane per mask word: two of a 4^3 leaf, four of a block in an 8^3 one).
+// Returns whether this lane set a new one.
 template <int L>
-__device__ __forceinline__ bool set_touched(const DevGrid &g, const BinSort &s)
+__device__ __forceinline__ bool set_touched(const DevGrid &g, const int *slot, const uint32_t *bits, int n)
 {
-    const int lane = lane_id();
-    int bs;
-    uint32_t want;
-    long long word;
-    if (L == 4) {
-        if (lane >= 16) return false;
-        bs = s.slot[lane >> 1];
-        want = s.bits[lane];
-        word = (long long)bs * 2 + (lane & 1);
-    } else {
-        bs = s.slot[lane >> 2];
-        const uint32_t h = s.bits[lane >> 1] >> ((lane & 1) << 4);  // the plane's 16 bits, k fastest
-        want = ((h & 0xfu) | (h & 0xf0u) << 4 | (h & 0xf00u) << 8 | (h & 0xf000u) << 12) << ((bs & 1) << 2);
-        word = (long long)(bs >> 3) * 16 + ((bs & 4) + (lane & 3)) * 2 + (bs >> 1 & 1);
+    bool set = false;
+    for (int q = lane_id(); q < n * (L == 4 ? 2 : 4); q += 32) {
+        int bs;
+        uint32_t want;
+        long long word;
+        if (L == 4) {
+            bs = slot[q >> 1];
+            want = bits[q];
+            word = (long long)bs * 2 + (q & 1);
+        } else {
+            bs = slot[q >> 2];
+            const uint32_t h = bits[q >> 1] >> ((q & 1) << 4);  // the plane's 16 bits, k fastest
+            want = ((h & 0xfu) | (h & 0xf0u) << 4 | (h & 0xf00u) << 8 | (h & 0xf000u) << 12) << ((bs & 1) << 2);
+            word = (long long)(bs >> 3) * 16 + ((bs & 4) + (q & 3)) * 2 + (bs >> 1 & 1);
+        }
+        if (!want || bs < 0) continue;
+        uint32_t *mw = g.mask + word;
+        set |= (*(volatile uint32_t *)mw & want) != want && (atomicOr(mw, want) & want) != want;
     }
-    if (!want || bs < 0) return false;
-    uint32_t *mw = g.mask + word;
-    return (*(volatile uint32_t *)mw & want) != want && (atomicOr(mw, want) & want) != want;
+    return set;
 }
 
 // Cell of a particle outside the bin's cells, relative to o, in 10 bits a

@@ -67,7 +67,7 @@ def test_particle_transfers_on_every_device(lib, lg2, affine):
         assert a("sg_p2g_apic", x, v, C if affine else None, 10, 1.0, 0, 1) == 0
         assert a("sg_flush") == 0, lib.sg_last_error()
         assert lib.sg_g2p2g(a.h, b.h, x, v, 10, 0.1, 1, 1.0, 0, 1) == 0, lib.sg_last_error()
-        assert a.log("k_p2g_gather", "k_g2p2g") == [1, 1]
+        assert a.log("k_p2g_gather", "k_g2p2g") == [1, 2]  # two forms of G2P2G, the device picks one
         assert a("sg_destroy") == b("sg_destroy") == 0
     lib.fake_device(0)
 

@@ -53,7 +53,10 @@ struct AdvectArgs {
 // cells and 692 at 5 (k_advect: 405, 405 and 410; with the choice 355, 403 and
 // 405).  The results are the same either way, so a largest component left over
 // from an earlier packing costs time only.
-__device__ __forceinline__ bool steps_within_a_cell(const AdvectArgs &A) { return __uint_as_float(__ldg(A.vmax)) * fabsf(A.h) < 1.f; }
+__device__ __forceinline__ bool steps_within_a_cell(const AdvectArgs &A)
+{
+    return __uint_as_float(__ldg(A.vmax)) * fabsf(A.h) < 1.f;
+}
 
 // Slot of the leaf holding cell (ci, cj, ck), relative to the list entry's
 // leaf (bi, bj, bk): through the neighbour table within one leaf, else the root.

@@ -48,7 +48,8 @@ struct Ctrl {
     int32_t never_set;    // a flag nothing writes (bounded-wait test)
     int32_t timeout_site; // which wait gave up (0 none, 1 look-back, 2 test, 3 leaf allocation)
                           // or, with kErrCheck, 100 + the failed check
-    int32_t bins_used;    // leaves holding particles in the last binned P2G
+    int32_t bins_used;    // bins with more than kFewParticles particles in the last binned P2G
+    int32_t bins_few;     // and bins with fewer
     long long act_total;  // active voxels of the last active-offset scan
     uint32_t rr_ticket;   // run-record tiles handed out (zeroed before each region-mask launch)
     int32_t moved[3];     // fused G2P2G over the last binning: particles found outside their bin's cells,
@@ -84,7 +85,8 @@ struct DevGrid {
     int32_t *perm;
     int32_t *perm_alt;  // the next binning's order, built from the last one (then swapped)
     int32_t *perm_key;    // each particle's bin, stored by the count pass for the order pass
-    int32_t *bin_list;  // the leaves holding particles, in no particular order
+    int32_t *bin_list;  // the bins holding particles, in no particular order: bins_used from
+                        // the front, bins_few from the back
     // grouped sweeps of the fused step: list entry of each slot (written by
     // the list generation), the records of runs of adjacent leaves (along i
     // for the column sweep, along j for the j-run sweep) bucketed by length,
@@ -285,6 +287,7 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
 // (p2g_words(R^3)), tile_sum (a word per kBinTile bin words), perm and
 // bin_list (p2g_bins).
 constexpr int kBinTile = 1024;
+constexpr int kFewParticles = 32;  // bins of so many can go by single warps (see sg_particle.cuh)
 __host__ __device__ constexpr long long p2g_bins(int R, int lg2) { return (long long)R * R * R << (3 * (lg2 - 2)); }
 __host__ __device__ constexpr long long p2g_words(long long bins) { return (bins + kBinTile) / kBinTile * kBinTile; }
 int p2g_launches(const DevGrid &g);  // kernels of one binned P2G

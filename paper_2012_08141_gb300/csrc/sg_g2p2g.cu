@@ -120,60 +120,6 @@ __device__ __forceinline__ bool scatter_node(const DevGrid &g, int i, int j, int
     return changed;
 }
 
-// P2G record of one particle: spline offsets and mass, q = m v - m dx C fx,
-// and the 9 entries of m dx C (row-major).
-struct P2GRec {
-    float4 r0, r1, r2, r3;
-};
-
-__device__ __forceinline__ P2GRec make_rec(float fx, float fy, float fz, float pmass, float3 u, const float (&c)[9],
-                                           float dx)
-{
-    float m[9];
-    const float md = pmass * dx;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) m[e] = md * c[e];
-    const float q0 = pmass * u.x - (m[0] * fx + m[1] * fy + m[2] * fz);
-    const float q1 = pmass * u.y - (m[3] * fx + m[4] * fy + m[5] * fz);
-    const float q2 = pmass * u.z - (m[6] * fx + m[7] * fy + m[8] * fz);
-    P2GRec r;
-    r.r0 = make_float4(fx, fy, fz, pmass);
-    r.r1 = make_float4(q0, q1, q2, m[0]);
-    r.r2 = make_float4(m[1], m[2], m[3], m[4]);
-    r.r3 = make_float4(m[5], m[6], m[7], m[8]);
-    return r;
-}
-
-// Node-by-node APIC P2G of one particle into g (slow path).
-__device__ __forceinline__ bool scatter_particle(const DevGrid &g, Spline sx, Spline sy, Spline sz, P2GRec r,
-                                                 int f_mass, int f_mom0)
-{
-    bool changed = false;
-    const int N = g.N;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int i = sx.base + a;
-        if ((unsigned)i >= (unsigned)N) continue;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int j = sy.base + b;
-            if ((unsigned)j >= (unsigned)N) continue;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const int k = sz.base + c;
-                if ((unsigned)k >= (unsigned)N) continue;
-                const float w = sx.w[a] * sy.w[b] * sz.w[c];
-                const float ta = (float)a, tb = (float)b, tc = (float)c;
-                const float u0 = fmaf(r.r1.w, ta, fmaf(r.r2.x, tb, fmaf(r.r2.y, tc, r.r1.x)));
-                const float u1 = fmaf(r.r2.z, ta, fmaf(r.r2.w, tb, fmaf(r.r3.x, tc, r.r1.y)));
-                const float u2 = fmaf(r.r3.y, ta, fmaf(r.r3.z, tb, fmaf(r.r3.w, tc, r.r1.z)));
-                changed |= scatter_node(g, i, j, k, w * r.r0.w, w * u0, w * u1, w * u2, f_mass, f_mom0);
-            }
-        }
-    }
-    return changed;
-}
-
 // ---------------------------------------------------------------------------
 // Sorting and summing of a chunk's new positions, in two forms.  Particles move
 // on from step to step and one binning serves many, so at first nearly all are
@@ -189,19 +135,21 @@ __device__ __forceinline__ bool scatter_particle(const DevGrid &g, Spline sx, Sp
 //                      onto the 8^3 nodes o - 1 .. o + 6.
 // Each launch counts the particles that it finds outside the own cells; from the
 // next launch over the same binning on, the second form runs if they were more
-// than one in kMovedShare.  Both are launched and the other returns at once.  2M
-// particles, 10 a cell, that have moved by 0 / 0.03 / 0.1 / 0.25 / 1 cell since
-// the binning: the first form takes 232 / 272 / 344 / 459 / 941 us, the second
-// (more shared memory, less L1) 257 / 302 / 342 / 349 / 347.
+// than one in kMovedShare and the bins hold more than kMovedBin each on average.
+// Both are launched and the other returns at once.  2M particles, 10 a cell, that
+// have moved by 0 / 0.03 / 0.1 / 0.25 / 1 cell since the binning: the first form
+// takes 232 / 272 / 344 / 459 / 941 us, the second (more shared memory, less L1)
+// 257 / 302 / 342 / 349 / 347.  200k, 3 a cell (192 a bin), moved by 0.25 / 1:
+// 103 / 156 and 107 / 106 us; one a cell (64 a bin): 174 / 233 and 239 / 287.
 // ---------------------------------------------------------------------------
-constexpr int kMovedShare = 16;
+constexpr int kMovedShare = 16, kMovedBin = 128;
 constexpr int kOwnCells = 64, kFarCell = 216, kFewMoved = 24;
 constexpr int kMovedBuf = 36 * 9 * 8;  // float4 [column][lane][node]
 
 struct MovedSort {
     int cnt[kFarCell + 1];    // particles per cell; zero between chunks
     int start[224];           // their places in idx
-    uint32_t prev[36], all[36];  // nodes that the particles of each column (6 x 6, of six cells) reach, before / after this chunk
+    uint32_t prev[36], all[36];  // nodes reached by each column's particles (6 x 6, of six cells), before / after this chunk
     int slot[8 + 27];         // blocks o / 4 + {0, 1}^3 and, for moved particles, o / 4 + {-1, 0, 1}^3
     uint32_t bits[2 * (8 + 27)]; // touched nodes of those blocks, i, j, k in order
     int moved;                // this chunk is summed by the 36 columns
@@ -418,27 +366,116 @@ struct G2P2GSmem {
     std::conditional_t<AROUND, MovedSort, BinSort> sort;
 };
 
-// One particle node by node: its G2P from src, its state, its P2G into dst.
-// Returns whether dst's structure changed.
-__device__ __noinline__ bool far_particle(const DevGrid &src, const DevGrid &dst, float *x, float *v, long long p,
-                                          float dt, int f_vel0, float pmass, int f_mass, int f_mom0)
+// One particle by a warp, node by node: its G2P from src, its state, its P2G
+// into dst.  Returns whether dst's structure changed.
+template <int L>
+__device__ __noinline__ bool far_particle(const DevGrid &src, const DevGrid &dst, float *x, float *v, long long p, float dt,
+                                          int f_vel0, float pmass, int f_mass, int f_mom0)
 {
-    const float x0 = x[3 * p], x1 = x[3 * p + 1], x2 = x[3 * p + 2];
-    float3 u;
-    float c[9];
-    g2p_from_grid<true>(src, src.field[f_vel0], src.field[f_vel0 + 1], src.field[f_vel0 + 2], bspline(x0, src.N),
-                        bspline(x1, src.N), bspline(x2, src.N), u, c);
-    const float n0 = x0 + dt * u.x, n1 = x1 + dt * u.y, n2 = x2 + dt * u.z;
-    v[3 * p] = u.x;
-    v[3 * p + 1] = u.y;
-    v[3 * p + 2] = u.z;
-    x[3 * p] = n0;
-    x[3 * p + 1] = n1;
-    x[3 * p + 2] = n2;
-    const Spline nx = bspline(n0, dst.N), ny = bspline(n1, dst.N), nz = bspline(n2, dst.N);
-    return scatter_particle(dst, nx, ny, nz, make_rec(nx.fx, ny.fx, nz.fx, pmass, u, c, 1.f / (float)dst.N), f_mass, f_mom0);
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, c = lane % 3, N = dst.N;
+    float xp[3], u[3], C[9];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) xp[e] = x[3 * p + e];
+    g2p_by_warp<L, true>(src, src.field[f_vel0], src.field[f_vel0 + 1], src.field[f_vel0 + 2], xp[0], xp[1], xp[2], u, C);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) xp[e] += dt * u[e];
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            v[3 * p + e] = u[e];
+            x[3 * p + e] = xp[e];
+        }
+    }
+    FewParticle<true> r;
+    few_particle<true>(r, xp[0], xp[1], xp[2], u, C, N);
+    const int i = r.b[0] + a, j = r.b[1] + b, k = r.b[2] + c;
+    if (lane >= 27 || (unsigned)i >= (unsigned)N || (unsigned)j >= (unsigned)N || (unsigned)k >= (unsigned)N) return false;
+    const float4 t = few_node<true>(r, a, b, c);
+    return scatter_node(dst, i, j, k, pmass * t.x, pmass * t.y, pmass * t.z, pmass * t.w, f_mass, f_mom0);
 }
 constexpr int kFar = -2;
+
+// The bins of few particles, a warp each (cf. the binned P2G): G2P, then the
+// sums of their new positions.  s: the CTA's scratch (kBinNodes + kFewScratch a
+// warp).
+template <int L>
+__device__ __noinline__ bool g2p2g_few(const DevGrid &src, const DevGrid &dst, const BinSplit &bins, const int32_t *bin_list,
+                                       const int32_t *bin_off, const int32_t *bin_end, const int32_t *perm, float *x, float *v,
+                                       float dt, int f_vel0, float pmass, int f_mass, int f_mom0, float4 *s)
+{
+    const int R = src.R, N = src.N, lane = lane_id(), warp = threadIdx.x >> 5;
+    bool changed = false;
+    float4 *s_u = s + warp * (kBinNodes + kFewScratch);
+    s = s_u + kBinNodes;
+    for (int w = blockIdx.x * kBinWarps + warp; w < bins.few; w += gridDim.x * kBinWarps) {
+        const int b = bin_list[bins.last - w], beg = bin_off[b], cnt = bin_end[b] - beg;
+        int bi, bj, bk;
+        bin_block<L>(b, R, bi, bj, bk);
+        const long long p = lane < cnt ? perm[beg + lane] : -1;
+        float xp[3] = {}, vp[3] = {}, cp[9] = {};
+        if (p >= 0) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) xp[e] = x[3 * p + e];
+        }
+        g2p_of_bin<L, true>(src, src.field[f_vel0], src.field[f_vel0 + 1], src.field[f_vel0 + 2], bi, bj, bk, cnt, xp, s_u, vp,
+                            cp);
+        FewParticle<true> r{};
+        if (p >= 0) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                xp[e] += dt * vp[e];
+                v[3 * p + e] = vp[e];
+                x[3 * p + e] = xp[e];
+            }
+            few_particle<true>(r, xp[0], xp[1], xp[2], vp, cp, N);
+        }
+        const unsigned strays = few_sums<true>(r, cnt, 4 * bi, 4 * bj, 4 * bk, s);
+        // the touched blocks' leaves, then the touched nodes' sums
+        uint32_t hits = 0, blocks = 0;
+#pragma unroll
+        for (int h = 0; h < 7; ++h) {
+            const int nd = h * 32 + lane;
+            int i, j, k, blk, l;
+            bin_node(nd, i, j, k, blk, l);
+            if (nd < kBinNodes && 4 * bi + i < N && 4 * bj + j < N && 4 * bk + k < N && few_hit(s, i, j, k)) {
+                hits |= 1u << h;
+                blocks |= 1u << blk;
+            }
+        }
+        blocks = __reduce_or_sync(kFull, blocks);
+        int slot = -1;
+        if (blocks >> lane & 1u) {
+            const int ci = bi + (lane >> 2), cj = bj + ((lane >> 1) & 1), ck = bk + (lane & 1);
+            bool fresh = false;
+            slot = block_of_leaf<L>(ensure_leaf(dst, block_leaf<L>(R, ci, cj, ck), fresh), ci, cj, ck);
+            changed |= fresh;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 7; ++h) {
+            const int nd = h * 32 + lane;
+            int i, j, k, blk, l;
+            bin_node(nd, i, j, k, blk, l);
+            const int bs = __shfl_sync(kFull, slot, blk & 7);
+            if (!(hits >> h & 1u) || bs < 0) continue;  // pool exhausted; the error is latched
+            const float4 t = s[nd];
+            const long long idx = block_voxel<L>(bs, i & 3, j & 3, k & 3);
+            changed |= set_bit(dst, idx);
+            atomicAdd(dst.field[f_mass] + idx, pmass * t.x);
+            atomicAdd(dst.field[f_mom0] + idx, pmass * t.y);
+            atomicAdd(dst.field[f_mom0 + 1] + idx, pmass * t.z);
+            atomicAdd(dst.field[f_mom0 + 2] + idx, pmass * t.w);
+        }
+        // the others, most of whose leaves are there now
+        few_strays<true>(r, strays, [&](int i, int j, int k, const float4 &t) {
+            if ((unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N && (unsigned)k < (unsigned)N)
+                changed |= scatter_node(dst, i, j, k, pmass * t.x, pmass * t.y, pmass * t.z, pmass * t.w, f_mass, f_mom0);
+        });
+        __syncwarp();  // s is cleared for the next bin
+    }
+    return changed;
+}
 
 template <int L, bool AROUND>
 __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant__ DevGrid src,
@@ -451,7 +488,9 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
     chained_entry();
     // of the three counts one is the last launch's, one this one's and one the
     // next one's, zero then
-    if ((bin_ctrl->moved[turn] > n / kMovedShare) != AROUND) return;
+    const bool many = bin_ctrl->moved[turn] > n / kMovedShare &&
+                      n > (long long)kMovedBin * (bin_ctrl->bins_used + bin_ctrl->bins_few);
+    if (many != AROUND) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) bin_ctrl->moved[(turn + 2) % 3] = 0;
     int moved_here = 0;
     using S = G2P2GSmem<AROUND>;
@@ -465,19 +504,26 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
     float *words = s.words[warp];
     const float *u0p = src.field[f_vel0], *u1p = src.field[f_vel0 + 1], *u2p = src.field[f_vel0 + 2];
     bool changed = false;
-    const int used = bin_ctrl->bins_used;
+    const BinSplit bins = bin_split(bin_ctrl, R, L, 0, 12);
+    const int used = bins.all;
     // particles whose stencil missed the domain when they were binned
     {
-        const int oob_bin = (int)p2g_bins(R, L == 8 ? 3 : 2);
+        const int oob_bin = bins.last + 1;
         const int end = bin_end[oob_bin];
-        for (int q = bin_off[oob_bin] + blockIdx.x * kBinThreads + threadIdx.x; q < end; q += gridDim.x * kBinThreads) {
-            changed |= far_particle(src, dst, x, v, perm[q], dt, f_vel0, pmass, f_mass, f_mom0);
-        }
+        for (int q = bin_off[oob_bin] + blockIdx.x * kBinWarps + warp; q < end; q += gridDim.x * kBinWarps)
+            changed |= far_particle<L>(src, dst, x, v, perm[q], dt, f_vel0, pmass, f_mass, f_mom0);
     }
-    int bl = blockIdx.x;
-    if (bl < used) {
+    // of a bin that several CTAs share, this one takes chunks part, part + parts, ...
+    const int parts = bins.parts, part = parts > 1 ? blockIdx.x / used : 0;
+    int bl = blockIdx.x - part * used, b = 0, beg = 0, end = 0;
+    if (bl < used && part < parts) {
+        b = nth_bin(bin_list, bins, bl);
+        beg = bin_off[b];
+        end = bin_end[b];
+    }
+    if (part * CAP < end - beg) {
         auto bin_of = [&](int l, int &b, int &beg, int &end) {
-            b = bin_list[l];
+            b = nth_bin(bin_list, bins, l);
             beg = bin_off[b];
             end = bin_end[b];
         };
@@ -510,11 +556,10 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                 }
             }
         };
-        int b, beg, end, nb = 0, nbeg = 0, nend = 0;
-        bin_of(bl, b, beg, end);
-        int slot = near_slot(b), c = 0, nch = (end - beg + CAP - 1) / CAP;
+        int nb = 0, nbeg = 0, nend = 0;
+        int slot = near_slot(b), c = part, nch = (end - beg + CAP - 1) / CAP;
         int p[PPT], pn[PPT];
-        order(beg, end, 0, nch, p);
+        order(beg, end, c, nch, p);
         request(p);
         if (bl + (int)gridDim.x < used) bin_of(bl + gridDim.x, nb, nbeg, nend);
         constexpr int OUT = AROUND ? kFarCell : kOwnCells;  // the cell of the particles that no column sums
@@ -529,14 +574,14 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
         if (threadIdx.x < 27) s.uslot[threadIdx.x] = slot;
         __syncthreads();
         for (;;) {
-            const bool last = c + 1 >= nch, more = !last || bl + (int)gridDim.x < used;
+            const bool last = c + parts >= nch, more = !last || bl + (int)gridDim.x < used;
             const int nnch = last ? (nend - nbeg + CAP - 1) / CAP : nch;
-            if (more) order(last ? nbeg : beg, last ? nend : end, last ? 0 : c + 1, nnch, pn);
+            if (more) order(last ? nbeg : beg, last ? nend : end, last ? 0 : c + parts, nnch, pn);
             if (last && more) slot = near_slot(nb);
             int bi, bj, bk;
             bin_block<L>(b, R, bi, bj, bk);
             const int oi = bi * 4, oj = bj * 4, ok = bk * 4;
-            if (c == 0) {  // src's node velocities, 0 outside the domain or the leaves
+            if (c == part) {  // src's node velocities, 0 outside the domain or the leaves
                 for (int nd = threadIdx.x; nd < 512; nd += kBinThreads) {
                     const int i = (nd >> 6) + 3, j = ((nd >> 3) & 7) + 3, k = (nd & 7) + 3;  // from o - 4
                     const int us = s.uslot[(i >> 2) * 9 + (j >> 2) * 3 + (k >> 2)];
@@ -619,7 +664,8 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
             } else {
                 bin_columns<true, CAP>(s.rec, s.idx, s.sort, s.buf);
             }
-            for (int pp = s.sort.start[moved ? OUT : kOwnCells] + warp; pp < s.sort.start[OUT + 1] && pp < CAP; pp += kBinWarps) {
+            for (int pp = s.sort.start[moved ? OUT : kOwnCells] + warp; pp < s.sort.start[OUT + 1] && pp < CAP;
+                 pp += kBinWarps) {
                 int i, j, k;
                 float4 t;
                 const int q = s.idx[pp];
@@ -631,7 +677,9 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
             }
 #pragma unroll
             for (int u = 0; u < PPT; ++u)
-                if (place[u] == kFar) changed |= far_particle(src, dst, x, v, p[u], dt, f_vel0, pmass, f_mass, f_mom0);
+                for (unsigned far = __ballot_sync(kFull, place[u] == kFar); far; far &= far - 1)
+                    changed |= far_particle<L>(src, dst, x, v, __shfl_sync(kFull, p[u], __ffs(far) - 1), dt, f_vel0, pmass,
+                                               f_mass, f_mom0);
             if (last) {
                 __syncthreads();
                 // the touched nodes' sums, then the dst leaves that hold them
@@ -722,7 +770,7 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
                 c = 0;
                 if (bl + (int)gridDim.x < used) bin_of(bl + gridDim.x, nb, nbeg, nend);
             } else {
-                ++c;
+                c += parts;
                 __syncthreads();  // the records are rewritten by the bin's next chunk
             }
             nch = nnch;
@@ -731,6 +779,10 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
         }
     }
     if (moved_here) atomicAdd(&bin_ctrl->moved[(turn + 1) % 3], moved_here);
+    static_assert(kBinWarps * (kBinNodes + kFewScratch) <= 4 * CAP, "the bins of few particles use the records' memory");
+    if (bins.few)
+        changed |= g2p2g_few<L>(src, dst, bins, bin_list, bin_off, bin_end, perm, x, v, dt, f_vel0, pmass, f_mass, f_mom0,
+                                s.rec[0]);
     if (changed) mark_dirty(dst);
 }
 

@@ -78,14 +78,47 @@ __global__ void __launch_bounds__(256) k_g2p(DevGrid g, float *__restrict__ x, f
     }
 }
 
+// The bins of few particles, a warp each (w: this warp among `warps`; s: its
+// scratch of kBinNodes).
+template <int L, bool APIC>
+__device__ __noinline__ void g2p_few(const DevGrid &g, const BinSplit &bins, float *x, float *v, float *C, float dt, int f_mom0,
+                                     int w, int warps, float4 *s)
+{
+    const int lane = lane_id();
+    for (; w < bins.few; w += warps) {
+        const int b = g.bin_list[bins.last - w], beg = g.bin_off[b], cnt = g.bin_count[b] - beg;
+        int bi, bj, bk;
+        bin_block<L>(b, g.R, bi, bj, bk);
+        const long long p = lane < cnt ? g.perm[beg + lane] : -1;
+        float xp[3] = {}, u[3] = {}, c[9] = {};
+        if (p >= 0) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) xp[e] = x[3 * p + e];
+        }
+        g2p_of_bin<L, APIC>(g, g.field[f_mom0], g.field[f_mom0 + 1], g.field[f_mom0 + 2], bi, bj, bk, cnt, xp, s, u, c);
+        if (p >= 0) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                v[3 * p + e] = u[e];
+                x[3 * p + e] = xp[e] + dt * u[e];
+            }
+            if (APIC) {
+#pragma unroll
+                for (int e = 0; e < 9; ++e) C[9 * p + e] = c[e];
+            }
+        }
+    }
+}
+
 // G2P over the bins of the last binned P2G: per bin, the node velocities of
 // the 6^3 nodes from o to o + 5 (o the bin's first node; every node a stencil
 // with base in [o, o + 3] reaches) are staged in shared memory, 0 outside the
 // domain or the allocated leaves, and the bin's particles read their 27 nodes
-// there.  A particle whose base lies outside that range (its
-// position changed since the binning, or a base of -2 / -1 at the low domain
-// face) reads the grid node by node, as do the particles whose stencil misses
-// the domain (the last bin).  A warp moves its particles' words together (see
+// there.  A particle whose base lies outside that range (its position changed
+// since the binning, or a base of -2 / -1 at the low domain face) reads the grid
+// node by node, as do the particles whose stencil misses the domain (the last
+// bin).  Bins of few particles go by warps, and several CTAs share a bin when
+// there are few bins (bin_split).  A warp moves its particles' words together (see
 // warp_fetch), positions one round ahead.  It waits on the bin's serial chain
 // (bin, order, positions; root, node values) and on the 27 shared 16-byte
 // reads a particle.  2M particles, about 10 a cell: 63 us, APIC 100k 11.5 us
@@ -93,25 +126,29 @@ __global__ void __launch_bounds__(256) k_g2p(DevGrid g, float *__restrict__ x, f
 // divisions per bin).  APIC at three CTAs per SM: at four its 9 words of C
 // spill (13.4 us).
 template <int L, bool APIC>
-__global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(DevGrid g, float *__restrict__ x, float *__restrict__ v,
-                                                       float *__restrict__ C, float dt, int f_mom0)
+__global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(const __grid_constant__ DevGrid g,
+                                                                  float *__restrict__ x, float *__restrict__ v,
+                                                                  float *__restrict__ C, float dt, int f_mom0)
 {
     chained_entry();
-    constexpr int B = 6, LG2 = L == 8 ? 3 : 2;
-    __shared__ float4 s_u[B * B * B];
-    __shared__ float s_words[8][32 * (APIC ? 9 : 3)];
-    float *s_t = s_words[threadIdx.x >> 5];
+    constexpr int B = 6;
+    __shared__ float4 s_raw[8 * kBinNodes];  // a bin's nodes and each warp's words, or a bin's nodes for each warp
+    float4 *s_u = s_raw;
+    float *s_t = reinterpret_cast<float *>(s_raw + kBinNodes) + (threadIdx.x >> 5) * (32 * (APIC ? 9 : 3));
     const int N = g.N, R = g.R;
     const float *f0 = g.field[f_mom0], *f1 = g.field[f_mom0 + 1], *f2 = g.field[f_mom0 + 2];
-    const int used = g.ctrl->bins_used;
-    const int oob_bin = R * R * R << (3 * (LG2 - 2));
-    // the next bin and its particle range are read a bin ahead
-    int nb = blockIdx.x < used ? g.bin_list[blockIdx.x] : oob_bin;
+    const BinSplit bins = bin_split(g.ctrl, R, L, 1, 4);
+    const int used = bins.all, oob_bin = bins.last + 1;
+    // this CTA's share of a bin that several take; the next bin and its particle
+    // range are read a bin ahead
+    const int part = bins.parts > 1 ? blockIdx.x / (used + 1) : 0, first = blockIdx.x - part * (used + 1);
+    int nb = first < used ? nth_bin(g.bin_list, bins, first) : oob_bin;
     int nbeg = g.bin_off[nb], nend = g.bin_count[nb];
-    for (int bl = blockIdx.x; bl <= used; bl += gridDim.x) {
-        const int b = nb, beg = nbeg, end = nend, next = bl + (int)gridDim.x;
+    for (int bl = part < bins.parts ? first : used + 1; bl <= used; bl += gridDim.x) {
+        const int b = nb, next = bl + (int)gridDim.x;
+        const unsigned beg = nbeg + 256u * part, end = nend;
         if (next <= used) {
-            nb = next < used ? g.bin_list[next] : oob_bin;
+            nb = next < used ? nth_bin(g.bin_list, bins, next) : oob_bin;
             nbeg = g.bin_off[nb];
             nend = g.bin_count[nb];
         }
@@ -122,7 +159,7 @@ __global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(DevGrid g, flo
         ok *= 4;
         // a warp's particles, 32 at a time; their positions are requested
         // before the staging barrier and one round ahead
-        int q = beg + (threadIdx.x & ~31) + lane_id();
+        unsigned q = beg + (threadIdx.x & ~31) + lane_id();
         int p = q < end ? g.perm[q] : -1;
         float t[3];
         warp_fetch<3>(x, p, t);
@@ -143,7 +180,7 @@ __global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(DevGrid g, flo
             float xp[3];
             warp_deal<3>(t, s_t, xp);
             const int cur = p;
-            q += blockDim.x;
+            q += blockDim.x * bins.parts;
             if (q - lane_id() < end) {
                 p = q < end ? g.perm[q] : -1;
                 warp_fetch<3>(x, p, t);
@@ -164,6 +201,9 @@ __global__ void __launch_bounds__(256, APIC ? 3 : 4) k_g2p_binned(DevGrid g, flo
         }
         __syncthreads();  // s_u is restaged for the next bin
     }
+    if (bins.few)
+        g2p_few<L, APIC>(g, bins, x, v, C, dt, f_mom0, blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8,
+                         s_raw + (threadIdx.x >> 5) * kBinNodes);
 }
 
 // CTAs of a persistent per-bin kernel: as many as fit on every SM at once.
@@ -260,7 +300,7 @@ __global__ void __launch_bounds__(256) k_bin_clear(DevGrid g)
     const long long q = blockIdx.x * 256LL + threadIdx.x;
     reinterpret_cast<int4 *>(g.bin_count)[q] = make_int4(0, 0, 0, 0);
     if (q < p2g_words(p2g_bins(g.R, 2)) / 4) reinterpret_cast<int4 *>(g.bin_reach)[q] = make_int4(0, 0, 0, 0);
-    if (q == 0) g.ctrl->bins_used = g.ctrl->moved[0] = g.ctrl->moved[1] = g.ctrl->moved[2] = 0;
+    if (q == 0) g.ctrl->bins_used = g.ctrl->bins_few = g.ctrl->moved[0] = g.ctrl->moved[1] = g.ctrl->moved[2] = 0;
 }
 
 // Particles of one bin with the reach classes `classes` (a bit each).  The
@@ -415,17 +455,20 @@ __global__ void __launch_bounds__(256) k_bin_place(DevGrid g, int alloc_ctas, bo
     // list of the bins with particles (the out-of-domain bin excluded)
     const int oob_bin = (int)p2g_bins(g.R, g.lg2);
     const int cnt[4] = {c4.x, c4.y, c4.z, c4.w};
-    int mine = 0;
+    int mine = 0;  // bins of more than kFewParticles, and in the upper half the others
 #pragma unroll
-    for (int q = 0; q < 4; ++q) mine += (cnt[q] > 0 && base + q < oob_bin) ? 1 : 0;
+    for (int q = 0; q < 4; ++q)
+        if (cnt[q] > 0 && base + q < oob_bin) mine += cnt[q] > kFewParticles ? 1 : 0x10000;
     const int upto = warp_incl_scan(mine), all = __shfl_sync(kFull, upto, 31);
     if (all) {
-        int first = 0;
-        if (lane == 31) first = atomicAdd(&g.ctrl->bins_used, all);
-        first = __shfl_sync(kFull, first, 31) + upto - mine;
+        int first = 0, few = 0;
+        if (lane == 31 && (all & 0xffff)) first = atomicAdd(&g.ctrl->bins_used, all & 0xffff);
+        if (lane == 31 && all >> 16) few = atomicAdd(&g.ctrl->bins_few, all >> 16);
+        first = __shfl_sync(kFull, first, 31) + (upto - mine & 0xffff);
+        few = oob_bin - 1 - (__shfl_sync(kFull, few, 31) + (upto - mine >> 16));
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (cnt[q] > 0 && base + q < oob_bin) g.bin_list[first++] = base + q;
+            if (cnt[q] > 0 && base + q < oob_bin) g.bin_list[cnt[q] > kFewParticles ? first++ : few--] = base + q;
     }
 }
 
@@ -476,8 +519,66 @@ struct GatherSmem {
     BinSort sort;
 };
 
+// The bins of few particles, a warp each; s: the CTA's scratch (kFewScratch a
+// warp).  Returns whether the structure changed.
 template <int L, bool APIC>
-__global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const float *__restrict__ x,
+__device__ __noinline__ bool gather_few(const DevGrid &g, const BinSplit &bins, const float *__restrict__ x, const float *__restrict__ v,
+                                        const float *__restrict__ C, float pmass, int f_mass, int f_mom0, float4 *s)
+{
+    const int R = g.R, N = g.N, lane = lane_id(), warp = threadIdx.x >> 5;
+    float *fm = g.field[f_mass], *f0 = g.field[f_mom0], *f1 = g.field[f_mom0 + 1], *f2 = g.field[f_mom0 + 2];
+    bool changed = false;
+    s += warp * kFewScratch;
+    auto add = [&](int bs, int i, int j, int k, const float4 &t) {
+        if (bs < 0) return;  // outside the domain, or the pool is exhausted (latched)
+        const long long idx = block_voxel<L>(bs, i & 3, j & 3, k & 3);
+        changed |= set_bit(g, idx);
+        atomicAdd(fm + idx, pmass * t.x);
+        atomicAdd(f0 + idx, pmass * t.y);
+        atomicAdd(f1 + idx, pmass * t.z);
+        atomicAdd(f2 + idx, pmass * t.w);
+    };
+    for (int w = blockIdx.x * kBinWarps + warp; w < bins.few; w += gridDim.x * kBinWarps) {
+        const int b = g.bin_list[bins.last - w], beg = g.bin_off[b], cnt = g.bin_count[b] - beg;
+        int bi, bj, bk;
+        bin_block<L>(b, R, bi, bj, bk);
+        const int slot = lane < 8 ? block_slot<L>(g.root, R, bi + (lane >> 2), bj + ((lane >> 1) & 1), bk + (lane & 1)) : -1;
+        FewParticle<APIC> r{};
+        long long p = -1;
+        if (lane < cnt) {
+            p = g.perm[beg + lane];
+            const float vp[3] = {v[3 * p], v[3 * p + 1], v[3 * p + 2]};
+            float c[9] = {};
+            if (APIC) {
+#pragma unroll
+                for (int e = 0; e < 9; ++e) c[e] = C[9 * p + e];
+            }
+            few_particle<APIC>(r, x[3 * p], x[3 * p + 1], x[3 * p + 2], vp, c, N);
+        }
+        // the cell order, which G2P reads
+        const int ri = r.b[0] - 4 * bi, rj = r.b[1] - 4 * bj, rk = r.b[2] - 4 * bk;
+        const int key = ((unsigned)(ri | rj | rk) < 4u ? (ri * 4 + rj) * 4 + rk : 64) << 5 | lane;
+        int rank = 0;
+        for (int t = 0; t < cnt; ++t) rank += __shfl_sync(kFull, key, t) < key;
+        if (lane < cnt) g.perm_alt[beg + rank] = (int)p;
+        const unsigned strays = few_sums<APIC>(r, cnt, 4 * bi, 4 * bj, 4 * bk, s);
+        for (int nd = lane; nd < 224; nd += 32) {
+            int i, j, k, blk, l;
+            bin_node(nd, i, j, k, blk, l);
+            const int bs = __shfl_sync(kFull, slot, blk & 7);
+            if (nd < kBinNodes && few_hit(s, i, j, k)) add(bs, i, j, k, s[nd]);
+        }
+        few_strays<APIC>(r, strays, [&](int i, int j, int k, const float4 &t) {
+            if ((unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N && (unsigned)k < (unsigned)N)
+                add(block_slot<L>(g.root, R, i >> 2, j >> 2, k >> 2), i, j, k, t);
+        });
+        __syncwarp();  // s is cleared for the next bin
+    }
+    return changed;
+}
+
+template <int L, bool APIC>
+__global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(const __grid_constant__ DevGrid g, const float *__restrict__ x,
                                                                const float *__restrict__ v,
                                                                const float *__restrict__ C, float pmass, int f_mass,
                                                                int f_mom0)
@@ -493,18 +594,22 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
     float *fm = g.field[f_mass];
     float *f0 = g.field[f_mom0], *f1 = g.field[f_mom0 + 1], *f2 = g.field[f_mom0 + 2];
     bool changed = false;
-    const int used = g.ctrl->bins_used;
+    const BinSplit bins = bin_split(g.ctrl, R, L, 0, 4);
+    const int used = bins.all;
     {   // the particles whose stencil misses the domain keep their order
-        const int oob_bin = (int)p2g_bins(R, L == 8 ? 3 : 2);
+        const int oob_bin = bins.last + 1;
         const int end = g.bin_count[oob_bin];
         for (int q = g.bin_off[oob_bin] + blockIdx.x * kBinThreads + threadIdx.x; q < end; q += gridDim.x * kBinThreads)
             g.perm_alt[q] = g.perm[q];
     }
-    int bl = blockIdx.x;
-    if (bl >= used) return;
+    static_assert(kBinWarps * kFewScratch <= S::NREC * CAP, "the bins of few particles use the records' memory");
+    auto few = [&] { return bins.few && gather_few<L, APIC>(g, bins, x, v, C, pmass, f_mass, f_mom0, s.rec[0]); };
+    // of a bin that several CTAs share, this one takes chunks part, part + parts, ...
+    const int parts = bins.parts, part = parts > 1 ? blockIdx.x / used : 0;
+    int bl = blockIdx.x - part * used;
     // a bin and its particle range; slot of its corner block (threads 0 .. 7)
     auto bin_of = [&](int l, int &b, int &beg, int &end) {
-        b = g.bin_list[l];
+        b = nth_bin(g.bin_list, bins, l);
         beg = g.bin_off[b];
         end = g.bin_count[b];
     };
@@ -545,11 +650,16 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
             }
         }
     };
-    int b, beg, end, nb = 0, nbeg = 0, nend = 0;
-    bin_of(bl, b, beg, end);
-    int slot = corner_slot(b), c = 0, nch = (end - beg + CAP - 1) / CAP;
+    int b, beg = 0, end = 0, nb = 0, nbeg = 0, nend = 0;
+    if (bl < used && part < parts) bin_of(bl, b, beg, end);
+    int c = part, nch = (end - beg + CAP - 1) / CAP;
+    if (c >= nch) {
+        if (few()) mark_dirty(g);
+        return;
+    }
+    int slot = corner_slot(b);
     int p[PPT], pn[PPT];
-    order(beg, end, 0, nch, p);
+    order(beg, end, c, nch, p);
     request(p);
     if (bl + (int)gridDim.x < used) bin_of(bl + gridDim.x, nb, nbeg, nend);
     if (threadIdx.x < 65) s.sort.cnt[threadIdx.x] = 0;
@@ -558,9 +668,9 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
     __syncthreads();
     for (;;) {
         // what comes after this chunk: the bin's next one, or the next bin
-        const bool last = c + 1 >= nch, more = !last || bl + (int)gridDim.x < used;
+        const bool last = c + parts >= nch, more = !last || bl + (int)gridDim.x < used;
         const int nnch = last ? (nend - nbeg + CAP - 1) / CAP : nch;
-        if (more) order(last ? nbeg : beg, last ? nend : end, last ? 0 : c + 1, nnch, pn);
+        if (more) order(last ? nbeg : beg, last ? nend : end, last ? 0 : c + parts, nnch, pn);
         if (last && more) slot = corner_slot(nb);
         int oi, oj, ok;
         bin_block<L>(b, R, oi, oj, ok);
@@ -651,13 +761,14 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(DevGrid g, const 
             c = 0;
             if (bl + (int)gridDim.x < used) bin_of(bl + gridDim.x, nb, nbeg, nend);
         } else {
-            ++c;
+            c += parts;
             __syncthreads();  // the records are rewritten by the bin's next chunk
         }
         nch = nnch;
 #pragma unroll
         for (int u = 0; u < PPT; ++u) p[u] = pn[u];
     }
+    changed |= few();
     if (changed) mark_dirty(g);
 }
 

@@ -518,4 +518,256 @@ __device__ __forceinline__ bool edge_node(const float4 (*rec)[CAP], int pp, int 
     return true;
 }
 
+// ---------------------------------------------------------------------------
+// Bins far emptier or fuller than a chunk.  Where the bins hold only a few
+// particles, the barriers and the fixed work of a CTA per bin are the whole time,
+// and those of up to kFewParticles go by a warp each: 200k particles, one in ten
+// cells, P2G on 4^3 / 8^3 leaves 353 / 354 -> 151 / 162 us (a CTA per whole leaf
+// had taken 397 / 181), G2P 106 / 109 -> 39 / 43, fused 787 / 800 -> 393 / 396.  A
+// launch with few such bins (up to `per_cta` for each of its CTAs) takes them like
+// the others: a warp alone needs longer for one than a CTA, and fused G2P2G, where
+// a particle that has left its bin costs the warp a step of its own, much longer
+// (200k particles in 3,600 bins, 1,500 of them such, moved by half a cell: 245 us,
+// all by CTAs 199; 200k in 10,500 such bins 291 and 399).
+// With at most half as many bins as CTAs, several share a bin, each with its
+// chunks of it: 1M particles in 61 bins, P2G 267 -> 116 us, G2P 124 -> 54.
+// ---------------------------------------------------------------------------
+
+// The bins of the last binned P2G as a launch takes them: `all` by CTAs (the
+// first `used` from the front of the list, the rest from its back), `parts` CTAs
+// to a bin, and the `few` others by warps.
+struct BinSplit {
+    int used, all, few, last, parts;
+};
+// extra: other work that a CTA takes like a bin.
+__device__ __forceinline__ BinSplit bin_split(const Ctrl *ctrl, int R, int L, int extra, int per_cta)
+{
+    BinSplit b;
+    const int few = ctrl->bins_few;
+    b.used = ctrl->bins_used;
+    b.few = few <= per_cta * (int)gridDim.x ? 0 : few;
+    b.all = b.used + few - b.few;
+    b.last = (int)p2g_bins(R, L == 8 ? 3 : 2) - 1;
+    const int n = b.all + extra;
+    b.parts = n > 0 && 2 * n <= (int)gridDim.x ? (int)gridDim.x / n : 1;
+    return b;
+}
+__device__ __forceinline__ int nth_bin(const int32_t *list, const BinSplit &b, int l)
+{
+    return list[l < b.used ? l : b.last - (l - b.used)];
+}
+
+// G2P of the particle at (x, y, z) (the same in all lanes) by a warp: lane (a,
+// b, c) < 27 reads its node from the grid (0 outside the domain or the leaves).
+template <int L, bool APIC>
+__device__ __forceinline__ void g2p_by_warp(const DevGrid &g, const float *f0, const float *f1, const float *f2, float x,
+                                            float y, float z, float (&u)[3], float (&c)[9])
+{
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, e = lane % 3, N = g.N;
+    const Spline sx = bspline(x, N), sy = bspline(y, N), sz = bspline(z, N);
+    float t[12] = {};
+    const int i = sx.base + a, j = sy.base + b, k = sz.base + e;
+    if (lane < 27 && (unsigned)i < (unsigned)N && (unsigned)j < (unsigned)N && (unsigned)k < (unsigned)N) {
+        const int bs = block_slot<L>(g.root, g.R, i >> 2, j >> 2, k >> 2);
+        if (bs >= 0) {
+            const long long idx = block_voxel<L>(bs, i & 3, j & 3, k & 3);
+            const float w = bs_eval(bs_poly(a), sx.fx) * bs_eval(bs_poly(b), sy.fx) * bs_eval(bs_poly(e), sz.fx);
+            const float wv[3] = {w * f0[idx], w * f1[idx], w * f2[idx]};
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                t[q] = wv[q];
+                if (APIC) {
+                    t[3 + 3 * q] = (float)a * wv[q];
+                    t[4 + 3 * q] = (float)b * wv[q];
+                    t[5 + 3 * q] = (float)e * wv[q];
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < (APIC ? 12 : 3); ++q) t[q] = warp_sum(t[q]);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) u[q] = t[q];
+    if (APIC) {
+        const float s4 = 4.f * (float)N, fx[3] = {sx.fx, sy.fx, sz.fx};
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int f = 0; f < 3; ++f) c[3 * q + f] = s4 * fmaf(-fx[f], u[q], t[3 + 3 * q + f]);
+    }
+}
+
+// G2P of the warp's particles (lanes 0 .. cnt - 1, positions x) of the bin of
+// block (bi, bj, bk): the bin's 6^3 nodes are staged in s, a particle that has
+// left the bin's cells goes by the whole warp.
+template <int L, bool APIC>
+__device__ __forceinline__ void g2p_of_bin(const DevGrid &g, const float *f0, const float *f1, const float *f2, int bi, int bj,
+                                           int bk, int cnt, const float (&x)[3], float4 *s, float (&u)[3], float (&c)[9])
+{
+    const int lane = lane_id(), N = g.N;
+    const int slot = lane < 8 ? block_slot<L>(g.root, g.R, bi + (lane >> 2), bj + ((lane >> 1) & 1), bk + (lane & 1)) : -1;
+#pragma unroll
+    for (int h = 0; h < 7; ++h) {
+        const int nd = h * 32 + lane;
+        int i, j, k, blk, l;
+        bin_node(nd, i, j, k, blk, l);
+        const int bs = __shfl_sync(kFull, slot, blk & 7);
+        if (nd >= kBinNodes) continue;
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (bs >= 0) {
+            const long long idx = block_voxel<L>(bs, i & 3, j & 3, k & 3);
+            t = make_float4(f0[idx], f1[idx], f2[idx], 0.f);
+        }
+        s[nd] = t;
+    }
+    __syncwarp();
+    const Spline sx = bspline(x[0], N), sy = bspline(x[1], N), sz = bspline(x[2], N);
+    const int ri = sx.base - 4 * bi, rj = sy.base - 4 * bj, rk = sz.base - 4 * bk;
+    const bool in = lane < cnt && (unsigned)ri < 4u && (unsigned)rj < 4u && (unsigned)rk < 4u;
+    if (in) {
+        float3 t;
+        g2p_from_block<6, APIC>(s, ri, rj, rk, N, sx, sy, sz, t, c);
+        u[0] = t.x;
+        u[1] = t.y;
+        u[2] = t.z;
+    }
+    for (unsigned stray = __ballot_sync(kFull, lane < cnt && !in); stray; stray &= stray - 1) {
+        const int t = __ffs(stray) - 1;
+        float us[3], cs[9];
+        g2p_by_warp<L, APIC>(g, f0, f1, f2, __shfl_sync(kFull, x[0], t), __shfl_sync(kFull, x[1], t),
+                             __shfl_sync(kFull, x[2], t), us, cs);
+        if (lane == t) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) u[e] = us[e];
+            if (APIC) {
+#pragma unroll
+                for (int e = 0; e < 9; ++e) c[e] = cs[e];
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// A lane's particle for P2G: base node, spline offsets, q = v - M f and M = dx C.
+template <bool APIC>
+struct FewParticle {
+    int b[3];
+    float f[3], q[3], m[APIC ? 9 : 1];
+};
+template <bool APIC>
+__device__ __forceinline__ void few_particle(FewParticle<APIC> &r, float x, float y, float z, const float (&v)[3],
+                                             const float (&C)[9], int N)
+{
+    const Spline sx = bspline(x, N), sy = bspline(y, N), sz = bspline(z, N);
+    r.b[0] = sx.base;
+    r.b[1] = sy.base;
+    r.b[2] = sz.base;
+    r.f[0] = sx.fx;
+    r.f[1] = sy.fx;
+    r.f[2] = sz.fx;
+    const float dx = 1.f / (float)N;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        r.q[e] = v[e];
+        if (APIC) {
+#pragma unroll
+            for (int f = 0; f < 3; ++f) r.m[APIC ? 3 * e + f : 0] = dx * C[3 * e + f];
+            r.q[e] -= r.m[APIC ? 3 * e : 0] * sx.fx + r.m[APIC ? 3 * e + 1 : 0] * sy.fx + r.m[APIC ? 3 * e + 2 : 0] * sz.fx;
+        }
+    }
+}
+
+// Its contribution (weight, weighted velocity) to node b + (a, b, c).
+template <bool APIC>
+__device__ __forceinline__ float4 few_node(const FewParticle<APIC> &r, int a, int b, int c)
+{
+    const float w = bs_eval(bs_poly(a), r.f[0]) * bs_eval(bs_poly(b), r.f[1]) * bs_eval(bs_poly(c), r.f[2]);
+    float u[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+        u[e] = APIC ? fmaf(r.m[APIC ? 3 * e : 0], (float)a,
+                           fmaf(r.m[APIC ? 3 * e + 1 : 0], (float)b, fmaf(r.m[APIC ? 3 * e + 2 : 0], (float)c, r.q[e])))
+                    : r.q[e];
+    return make_float4(w, w * u[0], w * u[1], w * u[2]);
+}
+
+// Lane t's particle, in every lane.
+template <bool APIC>
+__device__ __forceinline__ FewParticle<APIC> few_of(const FewParticle<APIC> &r, int t)
+{
+    FewParticle<APIC> o;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        o.b[e] = __shfl_sync(kFull, r.b[e], t);
+        o.f[e] = __shfl_sync(kFull, r.f[e], t);
+        o.q[e] = __shfl_sync(kFull, r.q[e], t);
+    }
+    if (APIC) {
+#pragma unroll
+        for (int e = 0; e < (APIC ? 9 : 1); ++e) o.m[e] = __shfl_sync(kFull, r.m[e], t);
+    }
+    return o;
+}
+
+// Scratch of a warp: the sums of the bin's 6^3 nodes, the occupied cells of its
+// 16 columns.
+constexpr int kFewScratch = kBinNodes + 4;  // float4
+
+// The sums, in s[node], of those of the warp's particles (lanes 0 .. cnt - 1)
+// whose base is in the bin's cells o .. o + 3; returns the lanes of the others.
+template <bool APIC>
+__device__ __forceinline__ unsigned few_sums(const FewParticle<APIC> &r, int cnt, int oi, int oj, int ok, float4 *s)
+{
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, c = lane % 3;
+    uint32_t *cells = reinterpret_cast<uint32_t *>(s + kBinNodes);
+    for (int q = lane; q < kBinNodes; q += 32) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (lane < 16) cells[lane] = 0;
+    const int ri = r.b[0] - oi, rj = r.b[1] - oj, rk = r.b[2] - ok;
+    const bool in = (unsigned)ri < 4u && (unsigned)rj < 4u && (unsigned)rk < 4u;
+    __syncwarp();
+    if (lane < cnt && in) atomicOr(&cells[ri * 4 + rj], 1u << rk);
+    for (unsigned ins = __ballot_sync(kFull, lane < cnt && in); ins; ins &= ins - 1) {
+        const FewParticle<APIC> o = few_of<APIC>(r, __ffs(ins) - 1);
+        const float4 add = few_node<APIC>(o, a, b, c);
+        if (lane < 27) {
+            float4 &n = s[((o.b[0] - oi + a) * 6 + o.b[1] - oj + b) * 6 + o.b[2] - ok + c];
+            n = make_float4(n.x + add.x, n.y + add.y, n.z + add.z, n.w + add.w);
+        }
+        __syncwarp();
+    }
+    return __ballot_sync(kFull, lane < cnt && !in);
+}
+
+// put(i, j, k, t) for each node of each of the others.
+template <bool APIC, typename F>
+__device__ __forceinline__ void few_strays(const FewParticle<APIC> &r, unsigned strays, F &&put)
+{
+    const int lane = lane_id(), a = lane / 9, b = (lane / 3) % 3, c = lane % 3;
+    for (; strays; strays &= strays - 1) {
+        const FewParticle<APIC> o = few_of<APIC>(r, __ffs(strays) - 1);
+        if (lane < 27) put(o.b[0] + a, o.b[1] + b, o.b[2] + c, few_node<APIC>(o, a, b, c));
+    }
+}
+
+// Does any of them hold bin node (i, j, k) in its stencil?
+__device__ __forceinline__ bool few_hit(const float4 *s, int i, int j, int k)
+{
+    const uint32_t *cells = reinterpret_cast<const uint32_t *>(s + kBinNodes);
+    uint32_t m = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            if ((unsigned)(i - a) <= 3u && (unsigned)(j - b) <= 3u) m |= cells[(i - a) * 4 + (j - b)];
+    return (((m | (m << 1) | (m << 2)) >> k) & 1u) != 0u;
+}
+
+// Set the bit of value index idx in the mask; whether it is new.
+__device__ __forceinline__ bool set_bit(const DevGrid &g, long long idx)
+{
+    uint32_t *mw = g.mask + (idx >> 5);
+    const uint32_t bit = 1u << (idx & 31);
+    return !(*(volatile uint32_t *)mw & bit) && !(atomicOr(mw, bit) & bit);
+}
+
 }  // namespace sg

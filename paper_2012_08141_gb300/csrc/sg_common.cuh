@@ -121,6 +121,12 @@ inline cudaError_t resident_per_sm(K *kernel, int threads, int bytes, std::atomi
 __device__ __forceinline__ void mark_dirty(const DevGrid &g) { *(volatile int32_t *)&g.ctrl->dirty = 1; }
 
 __device__ __forceinline__ void raise_error(const DevGrid &g, int bits) { atomicOr(&g.ctrl->err, bits); }
+// A kernel's check `site` of its own accesses failed.
+__device__ __forceinline__ void raise_check(const DevGrid &g, int site)
+{
+    raise_error(g, kErrCheck);
+    g.ctrl->timeout_site = 100 + site;
+}
 
 // ---------------------------------------------------------------------------
 // Allocation of the leaves marked in g.need.

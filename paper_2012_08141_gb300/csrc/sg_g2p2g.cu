@@ -37,15 +37,15 @@ namespace {
 constexpr int kRootPending = -2;  // a CTA is allocating this leaf
 constexpr int kRootFailed = -3;   // allocation failed (pool exhausted)
 
-// Self-checks of the kernel's own accesses: every vector access below first
-// verifies the alignment of its address (and the shared-record loop its
-// range); a failed check skips the access, latches kErrCheck on dst and
-// records which check failed.  They cost a few integer operations per access.
+// Self-checks of the kernel's own accesses; a failed one latches kErrCheck on
+// dst and records which it was (misaligned: also sort_fits, sg_particle.cuh).
+// Site 3: a new leaf's fields are zeroed in 16-byte stores, or, if not so
+// aligned, word by word.  Site 4: the base of the shared memory, whose records
+// move in 16-byte words (reported only: nothing could be done without it).
 __device__ __forceinline__ bool misaligned(const DevGrid &g, const void *p, unsigned align, int site)
 {
     if (((uintptr_t)p & (uintptr_t)(align - 1)) == 0) return false;
-    atomicOr(&g.ctrl->err, kErrCheck);
-    g.ctrl->timeout_site = 100 + site;
+    raise_check(g, site);
     return true;
 }
 
@@ -166,8 +166,9 @@ __device__ __forceinline__ int moved_cell(int i, int j, int k)
     return kOwnCells + ((unsigned)(i - 1) < 4u ? (j == 0 ? 72 : 96) + (i - 1) * 6 + k : (i == 0 ? 0 : 36) + j * 6 + k);
 }
 
-// Exclusive scan of the cell counts (one warp), which it zeroes.
-__device__ __forceinline__ void moved_scan(MovedSort &s)
+// Exclusive scan of the cell counts (one warp), which it zeroes; cap: the most
+// that there can be.
+__device__ __forceinline__ void moved_scan(const DevGrid &g, MovedSort &s, int cap)
 {
     constexpr int PER = 7;  // 32 x 7 >= 217; an odd stride has no bank conflicts
     const int lane = lane_id();
@@ -188,6 +189,7 @@ __device__ __forceinline__ void moved_scan(MovedSort &s)
     __syncwarp();
     const bool moved = s.start[kFarCell] - s.start[kOwnCells] > kFewMoved;
     if (lane == 0) {
+        sort_fits(g, s.start[kFarCell + 1], cap, 6);
         s.moved = moved;
         if (moved) s.outer = 1;
     }
@@ -645,8 +647,8 @@ __global__ void __launch_bounds__(kBinThreads, 2) k_g2p2g(const __grid_constant_
             }
             __syncthreads();
             if (warp == 0) {
-                if constexpr (AROUND) moved_scan(s.sort);
-                else bin_scan(s.sort);
+                if constexpr (AROUND) moved_scan(dst, s.sort, CAP);
+                else bin_scan(dst, s.sort, CAP);
             }
             __syncthreads();
             if (threadIdx.x == 0) moved_here += s.sort.start[OUT + 1] - s.sort.start[kOwnCells];

@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(const __grid_cons
             }
         }
         __syncthreads();
-        if (warp == 0) bin_scan(s.sort);
+        if (warp == 0) bin_scan(g, s.sort, CAP);
         __syncthreads();
         // the chunk's cell order (G2P reads it)
         const int first = beg + c * ((end - beg) / nch) + min(c, (end - beg) % nch);
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kBinThreads, 3) k_p2g_gather(const __grid_cons
         if (more) request(pn);
         bin_columns<APIC, CAP>(s.rec, s.idx, s.sort, s.buf);
         // bases -2 / -1 at the low domain faces: straight to the grid
-        for (int pp = s.sort.start[64] + warp; pp < s.sort.start[65]; pp += kBinWarps) {
+        for (int pp = s.sort.start[64] + warp; pp < s.sort.start[65] && pp < CAP; pp += kBinWarps) {
             int i, j, k;
             float4 t;
             if (!edge_node<APIC, CAP>(s.rec, s.idx[pp], oi, oj, ok, N, i, j, k, t)) continue;

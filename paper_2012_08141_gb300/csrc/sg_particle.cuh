@@ -276,8 +276,17 @@ struct BinSort {
     uint32_t bits[16]; // touched nodes of those blocks, i, j, k in order
 };
 
-// Exclusive scan of the cell counts (one warp), which it zeroes.
-__device__ __forceinline__ void bin_scan(BinSort &s)
+// A chunk's particles are at most cap: the loops over the sorted records take no
+// more (they would read past their memory), and a sort that counted more is an
+// error, or those left out would be lost without one.
+__device__ __forceinline__ void sort_fits(const DevGrid &g, int total, int cap, int site)
+{
+    if (total > cap) raise_check(g, site);
+}
+
+// Exclusive scan of the cell counts (one warp), which it zeroes; cap: the most
+// that there can be.
+__device__ __forceinline__ void bin_scan(const DevGrid &g, BinSort &s, int cap)
 {
     const int lane = lane_id();
     int c[4] = {0, 0, 0, 0};
@@ -302,6 +311,7 @@ __device__ __forceinline__ void bin_scan(BinSort &s)
         s.prev[lane] = before;
         s.all[lane] = before | now;
     } else if (lane == 16) {
+        sort_fits(g, run + tot, cap, 7);
         s.start[64] = run;
         s.start[65] = run + tot;
         s.cnt[64] = 0;

@@ -1012,8 +1012,8 @@ int do_flush(sg_grid *g)
                 rc = run_advect_run(g, i);
                 break;
             case OP_P2G:
-                if (capturing(g)) rc = bump_structure(g);  // refused before anything is recorded
-                if (!rc && !(rc = ensure_p2g_scratch(g, o.n))) {
+                if (capturing(g) && (rc = bump_structure(g))) break;  // refused before anything is recorded
+                if (!(rc = ensure_p2g_scratch(g, o.n))) {
                     // the same particles binned before: rebin from their last order,
                     // which is no longer one until all of the new one is launched
                     const bool rebin = g->p2g_x == o.p0 && g->p2g_n == o.n;
@@ -1044,8 +1044,8 @@ int do_flush(sg_grid *g)
                 ++i;
                 break;
             case OP_G2P2G:
-                if (capturing(g)) rc = bump_structure(g);  // refused before anything is recorded
-                if (!rc && !g->dry &&
+                if (capturing(g) && (rc = bump_structure(g))) break;  // refused before anything is recorded
+                if (!g->dry &&
                     (rc = cuda_check(launch_g2p2g(o.peer->dev, g->dev, o.bins->dev, g->stream, (float *)o.p1,
                                                   (float *)o.p2, o.n, o.f0, o.i0, o.f1, o.i1, o.i2,
                                                   o.bins->g2p2g_turn, g->lc),

@@ -55,7 +55,7 @@ struct AdvectArgs {
 // from an earlier packing costs time only.
 __device__ __forceinline__ bool steps_within_a_cell(const AdvectArgs &A)
 {
-    return __uint_as_float(*(const volatile uint32_t *)A.vmax) * fabsf(A.h) < 1.f;
+    return __uint_as_float(*A.vmax) * fabsf(A.h) < 1.f;
 }
 
 // Slot of the leaf holding cell (ci, cj, ck), relative to the list entry's

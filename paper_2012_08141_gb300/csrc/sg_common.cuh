@@ -51,9 +51,21 @@ __device__ __forceinline__ int warp_incl_scan(int v)
 // else, in every thread: it waits until the kernels before it have finished
 // and their writes are visible, and only then lets the next one come up (so at
 // most one waits).  After a copy, a memset or a kernel of another program the
-// launch is an ordinary one.  Between the kernels of a V-cycle the gap falls
-// from 2.1 us to none (ten cycles of the 512^3 band 1650 -> 1360 us, ten PIC
-// steps of 2M particles 3022 -> 2798 us, of 100k APIC particles 1008 -> 870 us).
+// launch is an ordinary one.  A kernel may be launched so only if chained_entry()
+// is its first statement: without the wait it would race with the one before it.
+//   Its CTAs are resident while the kernels before it still write what it reads.
+// For plain loads the wait is all that is needed.  __ldg and const __restrict__
+// become ld.global.nc, which wants data that do not change while the kernel reads
+// them: here, from the wait on.  That relies on two things: no such load moves
+// above the wait (a volatile asm that clobbers memory, as in
+// cudaGridDependencySynchronize(); each sits in a loop or behind a branch, and what
+// a kernel reads straight after the wait it reads with a plain load), and none is
+// served from a line cached before it.  The documented use of the wait works that
+// way, and a stale line would show in the tests that compare the bytes of long
+// runs; nothing that the kernel's own grid writes may be read through them.
+//   Between the kernels of a V-cycle the gap falls from 2.1 us to none (ten cycles
+// of the 512^3 band 1650 -> 1360 us, ten PIC steps of 2M particles 3022 -> 2798 us,
+// of 100k APIC particles 1008 -> 870 us).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void chained_entry()
 {
@@ -62,8 +74,8 @@ __device__ __forceinline__ void chained_entry()
 }
 
 template <typename... P, typename... A>
-inline cudaError_t launch_kernel(bool chained, void (*kernel)(P...), long long ctas, int threads, size_t smem, cudaStream_t s,
-                          A &&...args)
+inline cudaError_t launch_kernel(bool chained, void (*kernel)(P...), long long ctas, int threads, size_t smem,
+                                 cudaStream_t s, A &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ctas);

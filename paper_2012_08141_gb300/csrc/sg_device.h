@@ -281,8 +281,9 @@ void launch_sweep_single(const DevGrid &g, cudaStream_t s, int op, int src, int 
                          int sum_slot, const LaunchCfg &lc);
 
 // ---- particle kernels (sg_particle.cu) ----
-// Binned P2G (count, allocate, scan, order, accumulate per bin).  A bin is a 4^3 block of base nodes: a leaf, or
-// an eighth of an 8^3 leaf (numbered by leaf, then by octant).  Needs
+// Binned P2G (count, allocate, scan, order, accumulate per bin).  A bin is a 4^3
+// block of base nodes: a leaf, or an eighth of an 8^3 leaf (numbered by leaf, then
+// by octant).  Needs
 // bin_count / bin_off (p2g_words(p2g_bins) each), bin_reach
 // (p2g_words(R^3)), tile_sum (a word per kBinTile bin words), perm and
 // bin_list (p2g_bins).
@@ -300,16 +301,16 @@ cudaError_t launch_p2g_binned(DevGrid &g, cudaStream_t s, const float *x, const 
                               float pmass, int f_mass, int f_mom0, bool rebin, const LaunchCfg &lc);
 void launch_grid_update(const DevGrid &g, cudaStream_t s, int f_mass, int f_mom0, float dt,
                         float gz, int bound, const LaunchCfg &lc);
-// binned: use the bins of the last binned P2G over the same particles (the
-// particle order, leaf list and key ranges) to stage each leaf's
-// neighbourhood of node velocities in shared memory; otherwise input order.
-// C: NULL for PIC, else APIC, the matrices written there (n x 9 FP32).
 // The particle arrays (x, v: n x 3 FP32; C: n x 9 FP32; ids: n int64; any of
 // the last two may be null) permuted into the order g.perm of the last
 // binning, in place through tmp (n x 9 x 4 bytes), and g.perm reset to the
 // identity.  Returns the number of kernels launched.
 int launch_sort_particles(DevGrid &g, cudaStream_t s, float *x, float *v, float *C, int64_t *ids, long long n,
                           void *tmp, const LaunchCfg &lc);
+// binned: use the bins of the last binned P2G over the same particles (the
+// particle order, bin list and ranges) to stage each bin's nodes in shared
+// memory; otherwise input order.  C: NULL for PIC, else APIC, the matrices
+// written there (n x 9 FP32).
 void launch_g2p(const DevGrid &g, cudaStream_t s, float *x, float *v, float *C, long long n, float dt, int f_mom0,
                 int binned, const LaunchCfg &lc);
 

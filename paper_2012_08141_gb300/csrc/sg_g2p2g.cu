@@ -13,7 +13,7 @@
 //
 // Work split: one CTA per bin of the last binned P2G over these particles (a
 // 4^3 block of nodes from o with the particles whose base node was in it when
-// binned).
+// binned); bins far emptier or fuller than a chunk as bin_split says.
 //   1. stage src's velocities of nodes o-1 .. o+6 in shared memory;
 //   2. per particle: G2P from the staged block, store x', v'; count it in its
 //      new base cell and store its P2G record of the new position;

@@ -2,7 +2,8 @@
 // by the separate (sg_particle.cu) and the fused G2P2G (sg_g2p2g.cu)
 // kernels: the quadratic B-spline of a particle along one axis, G2P of one
 // particle from a staged block of node velocities or node by node from the
-// grid (PIC, or APIC with the matrix C), and the particle-array accessors.
+// grid (PIC, or APIC with the matrix C), the particle-array accessors, the sums
+// of a bin by columns of cells, and those of a bin of few particles by a warp.
 #pragma once
 #include "sg_common.cuh"
 

@@ -12,10 +12,10 @@ namespace sg {
 // Activation from the shell predicate.  Each lane of a warp tests one of up
 // to 32 consecutive root cells' bounding boxes against the band; the warp
 // then takes the cells that can meet it one at a time and builds their mask
-// words with one ballot per 32 voxels; the cells with active voxels and a
-// null pointer get new leaves (zero-filled in every field), and the words are
-// ORed into the leaves.  The predicate is
-// exact in 32-bit integers: |2i + 1 - N| < N <= 4096, so D < 3 * 4096^2 <
+// words (two rows a lane on 8^3 leaves, a ballot per 32 voxels on 4^3 ones); the
+// cells with active voxels and a null pointer get new leaves (zero-filled in every
+// field), and the words are ORed into the leaves.  The predicate is exact in
+// 32-bit integers: |2i + 1 - N| < N <= 4096, so D < 3 * 4096^2 <
 // 2^31, and lo2 / hi2 are clamped to [-1, 2^31 - 1] without changing it.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void axis_range(int i0, int L, int N, int &mn, int &mx)
